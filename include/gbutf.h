@@ -244,13 +244,14 @@ int gbu_per_string_loop(gbu_ctx *ctx, int op, const void *src, const uint64_t *o
                         const uint64_t *dst_off, gbu_result *results, gbu_stream stream);
 
 /* Launch geometry of a batched operation.  A CTA of warps_per_cta warps claims
- * strings_per_claim consecutive strings at a time; each warp takes one string at a time,
- * except that strings of at least long_bytes input bytes are handled afterwards by the whole
- * CTA (warps_per_cta x 512 bytes per step). */
+ * strings_per_claim consecutive strings at a time (more in a large batch, fewer in one that
+ * would leave SMs idle); a warp packs its share of them, 32 chunks of 16 bytes per step, except
+ * that strings of at least long_bytes input bytes are handled afterwards by the whole CTA
+ * (warps_per_cta x 512 bytes per step). */
 typedef struct {
   int32_t warps_per_cta;      /* 4, 8 or 16 (default 8) */
   uint32_t strings_per_claim; /* 1 .. 1024 (default 64) */
-  uint32_t long_bytes;        /* >= 512 (default 4096) */
+  uint32_t long_bytes;        /* >= 512 (default 16384) */
   float tuned_ms;             /* the tuner's best time for this geometry; 0 if set by hand */
 } gbu_batch_config;
 

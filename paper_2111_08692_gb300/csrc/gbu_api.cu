@@ -196,7 +196,10 @@ extern "C" gbu_ctx *gbu_create(int device, uint64_t max_units) {
     delete c;
     return nullptr;
   }
-  for (int m = 0; m < K_COUNT; ++m) c->batch_cfg[m] = gbu_batch_config{8, 64, 4096, 0};
+  // Strings from 16 KiB on go to a whole CTA: packed, one of them keeps a warp busy for 32 steps,
+  // and the CTA's narrow regions cost more per byte (a million log-normal strings, 8 -> 16 / 16 -> 8:
+  // 461 / 530 us with the line at 4 KiB, 412 / 476 at 8 KiB, 387 / 438 at 16 KiB, 401 / 457 at 32).
+  for (int m = 0; m < K_COUNT; ++m) c->batch_cfg[m] = gbu_batch_config{8, 64, 16384, 0};
   if (init_workspace(c) != GBU_OK) {
     cudaFree(c->states);
     cudaFree(c->ws);
@@ -644,11 +647,15 @@ static int batch_launch(gbu_ctx *c, int m, const gbu_batch_config &cfg, const vo
   bp.results = results;
   bp.lens = lens;
   bp.ws = c->ws;
+  // a batch with fewer claims than SMs is cut finer, down to a string per warp
   bp.grab = cfg.strings_per_claim;
+  const uint64_t fine = B / (uint64_t)c->num_sms;
+  if (fine < bp.grab) bp.grab = fine > (uint64_t)cfg.warps_per_cta ? (uint32_t)fine : (uint32_t)cfg.warps_per_cta;
+  if (bp.grab > cfg.strings_per_claim) bp.grab = cfg.strings_per_claim;
   bp.long_bytes = cfg.long_bytes;
   DeviceGuard g(c->device);
   uint64_t grid = (uint64_t)c->num_sms * (uint64_t)c->batch_blocks_per_sm[m][warps_index(cfg.warps_per_cta)];
-  const uint64_t claims = (B + cfg.strings_per_claim - 1) / cfg.strings_per_claim;
+  const uint64_t claims = (B + bp.grab - 1) / bp.grab;
   if (claims < grid) grid = claims;
   if (grid < 1) grid = 1;
   void *args[] = {(void *)&bp};

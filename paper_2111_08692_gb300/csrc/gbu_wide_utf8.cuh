@@ -38,6 +38,12 @@ namespace gbu {
 // Byte mask (0xFF where bit 7 of the byte of x is set).
 __device__ __forceinline__ uint32_t byte_mask(uint32_t x) { return prmt(x, 0u, 0xBA98u); }
 
+// Bits 4k .. 4k + 3 of m as bit 7 of each byte: bit j of the nibble times 1 << (7 + 7j) lands at bit
+// 8j + 7, and no two terms of the product meet.
+__device__ __forceinline__ uint32_t nibble_flags(uint32_t m, int k) {
+  return (((m >> (4 * k)) & 0xFu) * 0x10204080u) & 0x80808080u;
+}
+
 // The 16-bit word of position j (0..3) from the byte planes L and H.
 __device__ __forceinline__ uint32_t plane_word(uint32_t L, uint32_t H, int j) {
   return __byte_perm(L, H, (uint32_t)(j | ((4 + j) << 4)));
@@ -137,8 +143,11 @@ struct Utf8ToUtf16Wide {
   // H4: leading bytes C0-DF / E0-EF / F0-FF occur in the region or in bytes 1-3 of the word
   // before it (the code for an absent class is left out).  Each non-continuation byte takes the
   // place of one word (a four-byte leading byte of two), the count the count pass gave the lane.
-  template <bool H2, bool H3, bool H4>
-  __device__ __forceinline__ static uint32_t wconvert_fast(const uint32_t W[10], uint32_t sa) {
+  // NW: the words of the lane (W[1..NW]).  EXACT: the lane may hold bytes outside its string (m: one
+  // bit per byte inside) and other strings' words lie next to the lane's, so every word is stored
+  // under its predicate and a lane never writes past the words it counts.
+  template <bool H2, bool H3, bool H4, int NW = 8, bool EXACT = false>
+  __device__ __forceinline__ static uint32_t wconvert_fast(const uint32_t (&W)[NW + 2], uint32_t sa, uint32_t m = 0) {
     // with a single class present, every byte >= C0 is a leading byte of that class; without
     // H4 there is no byte >= F0
     constexpr bool ONE = (int)H2 + (int)H3 + (int)H4 == 1;
@@ -152,7 +161,7 @@ struct Utf8ToUtf16Wide {
       if (H4) pF = ONE ? pg : pE & (w << 3);
     }
 #pragma unroll
-    for (int k = 1; k <= 8; ++k) {
+    for (int k = 1; k <= NW; ++k) {
       const uint32_t w = W[k], wn = W[k + 1];
       const uint32_t s1 = w << 1;
       const uint32_t g = w & s1 & 0x80808080u;     // >= C0
@@ -218,17 +227,18 @@ struct Utf8ToUtf16Wide {
         H = (Hhs & M4) | (H & ~M4);
       }
       // stage the words (2 bytes per leading byte, 4 where it takes two words)
-      const uint32_t step = H4 ? (n >> 6) + (gF >> 6) : n >> 6;
+      const uint32_t lead = EXACT ? n & nibble_flags(m, k - 1) : n;
+      const uint32_t step = H4 ? (lead >> 6) + (gF >> 6) : lead >> 6;
       constexpr int FREE = H4 ? 1 : 2;  // the last word's positions that a leading byte always follows
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const uint32_t bit = 0x80u << (8 * j), ones = 0x01010101u >> (32 - 8 * j - (j == 0 ? 8 : 0));
         const uint32_t at = j == 0 ? sa : __dp4a(step, ones, sa);
-        if (k < 8 || j < FREE) sts_u16(at, plane_word(L, H, j));
-        else sts_u16_if(at, plane_word(L, H, j), n, bit);
+        if (!EXACT && (k < NW || j < FREE)) sts_u16(at, plane_word(L, H, j));
+        else sts_u16_if(at, plane_word(L, H, j), lead, bit);
         if (H4) sts_u16_if(at + 2, plane_word(Lls, Hls, j), gF, bit);
       }
-      if (k < 8) sa = __dp4a(step, 0x01010101u, sa);
+      if (k < NW) sa = __dp4a(step, 0x01010101u, sa);
     }
     return bad;
   }
