@@ -52,7 +52,7 @@ def sources_hash() -> str:
 
 
 # The sources each single-buffer kernel is compiled from (its device code), by operation.
-_STREAM = ["gbu_stream.cu", "gbu_chunk.cuh", "gbu_device.cuh"]
+_STREAM = ["gbu_stream.cu", "gbu_planes.cuh", "gbu_chunk.cuh", "gbu_device.cuh"]
 KERNEL_SOURCES = {
     "validate_utf8": _STREAM, "utf16_length_from_utf8": _STREAM,
     "validate_utf16le": _STREAM, "utf8_length_from_utf16le": _STREAM,

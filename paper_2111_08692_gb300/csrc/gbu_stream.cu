@@ -1,6 +1,8 @@
 // gbu_stream.cu -- read-only kernels: validate_utf8, utf16_length_from_utf8,
 // validate_utf16le, utf8_length_from_utf16le.
 //
+// UTF-8 validation has a kernel of its own (validate8_kernel: bit planes, 32 bytes per lane); the
+// others are modes of stream_kernel.
 // These never wait on another CTA, so they stream straight from global memory: each warp
 // owns 4 KB warp tiles (round-robin over all warps of the grid), issues all eight 16-byte
 // loads of a lane before using any (ld.global.nc, no L1 allocation), and takes each chunk's
@@ -14,6 +16,7 @@
 #include "gbu_chunk.cuh"
 #include "gbu_device.cuh"
 #include "gbu_kernels.h"
+#include "gbu_planes.cuh"
 
 namespace gbu {
 
@@ -54,7 +57,7 @@ __global__ void __launch_bounds__(STREAM_THREADS, stream_min_blocks<KMODE>()) st
   // the warp -- all warps read that one word, so reading it every tile would queue them on one
   // L2 slice -- by a load that overlaps the tile's own loads).  The smallest flagged chunk is
   // never skipped.
-  const bool early = (MODE == S_V8 || MODE == S_V16) && p.early_exit != 0;
+  const bool early = MODE == S_V16 && p.early_exit != 0;
   uint32_t known = 0xFFFFFFFFu;
   // after a tile: publish a flagged tile and stop, or take the refreshed snapshot
   uint32_t it = 0;  // tiles this warp has started
@@ -92,24 +95,41 @@ __global__ void __launch_bounds__(STREAM_THREADS, stream_min_blocks<KMODE>()) st
       pre = swap16x2(pre);
       post = swap16x2(post);
     }
-    if (MODE == S_V8 || MODE == S_L16) {
+    if ((MODE == S_L16 || MODE == S_L8) && fast) {
+      // a warp tile inside the buffer: no neighbouring words and no bounds (1 GiB of CJK, UTF-16
+      // length: 208 us with the shuffles of the general loop below, 156 without)
+      constexpr uint32_t UNITS = MODE == S_L16 ? 16u : 8u;  // units of an ASCII chunk
       uint32_t any = 0;
 #pragma unroll
       for (int r = 0; r < ST_ROUNDS; ++r) any |= v[r].x | v[r].y | v[r].z | v[r].w;
-      if (__all_sync(0xffffffffu, fast && (any & 0x80808080u) == 0)) {
-        // an all-ASCII warp tile: 16 units per chunk, and the only possible error is a
-        // leading byte just before the tile that wants continuation bytes in it (lane 0)
-        if (MODE == S_L16) {
-          total += 16 * ST_ROUNDS;
-        } else if (lane == 0) {
-          const Flags8 fp = classify8(pre);
-          const uint32_t req = __funnelshift_l(fp.geC0, 0u, 8) | __funnelshift_l(fp.geE0, 0u, 16) |
-                               __funnelshift_l(fp.geF0, 0u, 24);
-          if (req && (unsigned long long)t0 < err_pos) err_pos = (unsigned long long)t0;
-        }
-        if (early && stop_after_tile(wt, snap)) break;
+      if (__all_sync(0xffffffffu, (any & (MODE == S_L16 ? 0x80808080u : 0xFF80FF80u)) == 0)) {
+        total += UNITS * ST_ROUNDS;
         continue;
       }
+      // flags in bit 7 of each byte, summed by byte dot products (0x80 per flag)
+      uint32_t add = 0, sub = 0;
+#pragma unroll
+      for (int r = 0; r < ST_ROUNDS; ++r) {
+        const uint32_t Wd[4] = {v[r].x, v[r].y, v[r].z, v[r].w};
+        if (MODE == S_L16) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const uint32_t w = Wd[k], s1 = w * 2u;
+            add = __dp4a((~w | s1) & 0x80808080u, 0x01010101u, add);                          // not a continuation
+            add = __dp4a(w & s1 & (w * 4u) & (w * 8u) & 0x80808080u, 0x01010101u, add);       // >= F0
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < 4; k += 2) {  // the high and the low bytes of four words
+            const uint32_t hb = __byte_perm(Wd[k], Wd[k + 1], 0x7531), lb = __byte_perm(Wd[k], Wd[k + 1], 0x6420);
+            add = __dp4a((((hb & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | hb | lb) & 0x80808080u, 0x01010101u, add);  // >= 80
+            add = __dp4a((((hb & 0x78787878u) + 0x78787878u) | hb) & 0x80808080u, 0x01010101u, add);       // >= 800
+            sub = __dp4a(bytes_sur(hb), 0x01010101u, sub);
+          }
+        }
+      }
+      total += (MODE == S_L8 ? UNITS * ST_ROUNDS : 0u) + ((add - sub) >> 7);
+      continue;
     }
     if (MODE == S_V16 && fast) {
       // A warp tile inside the buffer: surrogate flags of every word's high byte first; a tile
@@ -144,9 +164,6 @@ __global__ void __launch_bounds__(STREAM_THREADS, stream_min_blocks<KMODE>()) st
       if (early && stop_after_tile(wt, snap)) break;
       continue;
     }
-    // UTF-8 validation: the rounds whose chunk of this lane holds an error; the first one gives
-    // the lane's error position after the tile (one test per tile instead of one per round)
-    uint32_t em = 0;
 #pragma unroll
     for (int r = 0; r < ST_ROUNDS; ++r) {
       const long long c = t0 + 512 * r + 16 * lane;
@@ -161,70 +178,6 @@ __global__ void __launch_bounds__(STREAM_THREADS, stream_min_blocks<KMODE>()) st
       W[0] = lane == 0 ? before : up;
       W[5] = lane == 31 ? after : down;
 
-      if (MODE == S_V8) {
-        // Three routes, chosen per warp region by the leading bytes it holds (and the word
-        // before it): without bytes >= E0 (Latin, Cyrillic and other one- and two-byte text) a
-        // byte must be a continuation byte exactly when the byte before it is >= C0, and only
-        // C0/C1 can break rules 4-6; without bytes >= F0 (CJK) the >= F0 flags and tests drop
-        // out; else all three lead flags.
-        uint32_t s1[5], geC0[5], hi3 = 0;
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-          s1[k] = W[k] << 1;
-          geC0[k] = W[k] & s1[k] & 0x80808080u;
-          hi3 |= geC0[k] & (W[k] << 2);
-        }
-        if (!__any_sync(0xffffffffu, hi3 != 0)) {
-          uint32_t err = 0;
-#pragma unroll
-          for (int k = 1; k <= 4; ++k) {
-            const uint32_t isC = W[k] & ~s1[k] & 0x80808080u;
-            err |= __funnelshift_l(geC0[k - 1], geC0[k], 8) ^ isC;
-            err |= geC0[k] & ~((W[k] & 0x3E3E3E3Eu) + 0x7F7F7F7Fu);  // C0, C1
-          }
-          em |= err ? 1u << r : 0u;
-          continue;
-        }
-        // No leading byte >= F0 in the region (CJK and other text of one to three bytes):
-        // structure by the >= C0 and >= E0 flags only (the region holds bytes E0-EF).
-        Flags8 g[5];
-        uint32_t hi4 = 0;
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-          g[k].geC0 = geC0[k];
-          g[k].geE0 = geC0[k] & (W[k] << 2);
-          g[k].geF0 = g[k].geE0 & (W[k] << 3);
-          g[k].isC = W[k] & ~s1[k] & 0x80808080u;
-          hi4 |= g[k].geF0;
-        }
-        if (!__any_sync(0xffffffffu, hi4 != 0)) {
-          uint32_t err = 0, c2 = 0;
-#pragma unroll
-          for (int k = 1; k <= 4; ++k) {
-            const uint32_t req = __funnelshift_l(g[k - 1].geC0, g[k].geC0, 8) |
-                                 __funnelshift_l(g[k - 1].geE0, g[k].geE0, 16);
-            err |= req ^ g[k].isC;
-            c2 |= g[k].geC0 & ~g[k].geE0;
-          }
-          err |= utf8_special_errors(W, g, __any_sync(0xffffffffu, c2 != 0), true, false);
-          em |= err ? 1u << r : 0u;
-          continue;
-        }
-        // leading bytes >= F0 occur in the region: all three flags
-        uint32_t err = 0, c2 = 0, c3 = 0;
-#pragma unroll
-        for (int k = 1; k <= 4; ++k) {
-          const uint32_t req = __funnelshift_l(g[k - 1].geC0, g[k].geC0, 8) |
-                               __funnelshift_l(g[k - 1].geE0, g[k].geE0, 16) |
-                               __funnelshift_l(g[k - 1].geF0, g[k].geF0, 24);
-          err |= req ^ g[k].isC;
-          c2 |= g[k].geC0 & ~g[k].geE0;
-          c3 |= g[k].geE0 & ~g[k].geF0;
-        }
-        err |= utf8_special_errors(W, g, __any_sync(0xffffffffu, c2 != 0), __any_sync(0xffffffffu, c3 != 0), true);
-        em |= err ? 1u << r : 0u;
-        continue;
-      }
       if (MODE == S_L16) {
         Flags8 f[5];
 #pragma unroll
@@ -250,14 +203,10 @@ __global__ void __launch_bounds__(STREAM_THREADS, stream_min_blocks<KMODE>()) st
         total += cnt;
       }
     }
-    if (MODE == S_V8 && em) {
-      const unsigned long long c = (unsigned long long)(t0 + 512 * (__ffs(em) - 1) + 16 * lane);
-      if (c < err_pos) err_pos = c;
-    }
     if (early && stop_after_tile(wt, snap)) break;
   }
 
-  const bool want_err = MODE == S_V8 || MODE == S_V16;
+  const bool want_err = MODE == S_V16;
   if (!fold_and_finish<STREAM_THREADS>(p, want_err ? err_pos : total, want_err, red, &is_last)) return;
   if (threadIdx.x == 0) {
     const unsigned long long key = *(volatile unsigned long long *)&p.ws->errkey;
@@ -266,11 +215,6 @@ __global__ void __launch_bounds__(STREAM_THREADS, stream_min_blocks<KMODE>()) st
       *p.len_out = tot;
     } else if (key == NO_ERROR) {
       write_result(p.result, GBU_OK, p.n);
-    } else if (MODE == S_V8) {
-      int32_t kind;
-      uint64_t off;
-      resolve_utf8_error(p.base + p.off0, p.n, (long long)key - (long long)p.off0, &kind, &off);
-      write_result(p.result, kind, off);
     } else {
       uint64_t off;
       resolve_utf16_error<BE>(reinterpret_cast<const uint16_t *>(p.base + p.off0), p.n,
@@ -281,9 +225,115 @@ __global__ void __launch_bounds__(STREAM_THREADS, stream_min_blocks<KMODE>()) st
   reset_workspace(p);
 }
 
+// UTF-8 validation: a warp streams 4 KiB warp tiles, four regions of 1 KiB, a lane 32 consecutive
+// bytes of each (one 256-bit load; the source base is rounded to 32 bytes), judged on bit planes
+// (gbu_planes.cuh).  A region without a byte >= 80 takes one vote.  Bound by HBM for ASCII, by the
+// integer pipe else (CJK: 76% busy, 180 warp instructions per KiB; the byte-wise routes before took
+// 280).  Each region's registers are loaded with the warp's next tile as soon as the region is
+// judged, so that three regions' judgement covers the load.  1 GiB of CJK: 440 us before (2.4
+// TB/s), 266 with all loads of a tile issued together, 261 so.
+constexpr int V8_REGIONS = (int)(WT_BYTES / 1024u);
+
+// The lane's 32 bytes at virtual position c (bytes outside the input read as zero).
+__device__ __forceinline__ void load_lane32(const Params &p, long long c, bool inside, uint32_t (&w)[8]) {
+  if (inside) {
+    ldg32_stream(p.base + c, w);
+  } else {
+    const uint4 a = load_chunk(p, c, false), b = load_chunk(p, c + 16, false);
+    w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
+    w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
+  }
+}
+
+__global__ void __launch_bounds__(STREAM_THREADS, 3) validate8_kernel(const Params p) {
+  __shared__ unsigned long long red[ST_WARPS];
+  __shared__ int is_last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long nw = (long long)gridDim.x * ST_WARPS;
+  const long long lo = p.off0, hi = (long long)p.vbytes;
+  auto inside = [&](long long t0) { return t0 - 4 >= lo && t0 + (long long)WT_BYTES + 4 <= hi; };
+  auto edge_word = [&](long long v, bool in) { return in ? ldg_word(p.base + v) : load_word_checked(p, v); };
+  unsigned long long err_pos = NO_ERROR;
+  // early exit as in stream_kernel
+  const bool early = p.early_exit != 0;
+  uint32_t known = 0xFFFFFFFFu, it = 0;
+  long long wt = (long long)blockIdx.x * ST_WARPS + warp;
+  uint32_t W[V8_REGIONS][8], pre = 0, post = 0;
+  if (wt < (long long)p.ntiles) {
+    const long long t0 = wt * WT_BYTES;
+    const bool in = inside(t0);
+#pragma unroll
+    for (int r = 0; r < V8_REGIONS; ++r) load_lane32(p, t0 + 1024 * r + 32 * lane, in, W[r]);
+    pre = edge_word(t0 - 4, in);
+    post = edge_word(t0 + WT_BYTES, in);
+  }
+  for (; wt < (long long)p.ntiles; wt += nw) {
+    const long long t0 = wt * WT_BYTES, t1 = t0 + nw * WT_BYTES;  // this tile, the warp's next one
+    if (early && (uint32_t)wt > known) break;  // uniform over the warp
+    uint32_t snap = 0xFFFFFFFFu;
+    if (early && lane == 0 && (it & 7u) == 0) snap = ld_relaxed_u32(&p.ws->stop_tile);
+    ++it;
+    const bool more = wt + nw < (long long)p.ntiles, in = inside(t1);
+    uint32_t em = 0;  // the regions whose bytes of this lane hold an error
+    // continuation bytes wanted in the lane's bytes of the next region by those of this one (used
+    // from lane 31, for lane 0), at first those wanted by the word before the tile
+    uint32_t pending = wanted_after(pre);
+#pragma unroll
+    for (int r = 0; r < V8_REGIONS; ++r) {
+      uint32_t any = 0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) any |= W[r][k];
+      if (__any_sync(0xffffffffu, (any & 0x80808080u) != 0 || (lane == 31 && pending != 0))) {
+        const uint32_t after = r + 1 < V8_REGIONS ? W[r + 1 < V8_REGIONS ? r + 1 : r][0] : post;
+        const uint32_t next = __shfl_sync(0xffffffffu, lane == 0 ? after : W[r][0], (lane + 1) & 31);
+        const uint32_t err = utf8_plane_errors(
+            W[r],
+            [&](uint32_t out) {
+              const uint32_t wanted = __shfl_sync(0xffffffffu, lane == 31 ? pending : out, (lane + 31) & 31);
+              pending = out;
+              return wanted;
+            },
+            next);
+        em |= err ? 1u << r : 0u;
+      } else {
+        pending = 0;
+      }
+      if (more) load_lane32(p, t1 + 1024 * r + 32 * lane, in, W[r]);
+    }
+    if (more) {
+      pre = edge_word(t1 - 4, in);
+      post = edge_word(t1 + WT_BYTES, in);
+    }
+    if (em) {
+      const unsigned long long c = (unsigned long long)(t0 + 1024 * (__ffs(em) - 1) + 32 * lane);
+      if (c < err_pos) err_pos = c;
+    }
+    if (early) {
+      if (__any_sync(0xffffffffu, err_pos != NO_ERROR)) {
+        if (lane == 0) atomicMin(&p.ws->stop_tile, (uint32_t)wt);
+        break;
+      }
+      if ((it & 7u) == 1u) known = __shfl_sync(0xffffffffu, snap, 0);
+    }
+  }
+  if (!fold_and_finish<STREAM_THREADS>(p, err_pos, true, red, &is_last)) return;
+  if (threadIdx.x == 0) {
+    const unsigned long long key = *(volatile unsigned long long *)&p.ws->errkey;
+    if (key == NO_ERROR) {
+      write_result(p.result, GBU_OK, p.n);
+    } else {
+      int32_t kind;
+      uint64_t off;
+      resolve_utf8_error(p.base + p.off0, p.n, (long long)key - (long long)p.off0, &kind, &off);
+      write_result(p.result, kind, off);
+    }
+  }
+  reset_workspace(p);
+}
+
 const void *stream_kernel_ptr(int mode) {
   switch (mode) {
-    case S_V8: return (const void *)stream_kernel<S_V8>;
+    case S_V8: return (const void *)validate8_kernel;
     case S_L16: return (const void *)stream_kernel<S_L16>;
     case S_V16: return (const void *)stream_kernel<S_V16>;
     case S_V16BE: return (const void *)stream_kernel<S_V16BE>;
