@@ -10,6 +10,7 @@
 #include "gbu_device.cuh"
 #include "gbu_internal.h"
 #include "gbu_kernels.h"
+#include "gbu_wide.cuh"
 #include "gbutf.h"
 
 namespace {
@@ -21,6 +22,7 @@ enum Kernel {
   K_V16BE = K_COUNT, K_L16BE, K_C16BE, K_C8BE,
   K_V32, K_L8F32, K_L32, K_C32, K_C8T32,  // validate, UTF-8 length, UTF-32 length, 32 -> 8, 8 -> 32
   K_L16F32, K_L32F16, K_C32T16, K_C16T32,  // UTF-16 length, UTF-32 length of UTF-16, 32 -> 16, 16 -> 32
+  K_C8S, K_C16S, K_C16BES, K_C8BES,        // K_C8, K_C16, K_C16BE, K_C8BE on small inputs (4 KiB partitions)
   K_ALL
 };
 
@@ -30,11 +32,11 @@ const void *kernel_ptr(int k) {
     case K_L8: return gbu::stream_kernel_ptr(1);
     case K_V16: return gbu::stream_kernel_ptr(2);
     case K_L16: return gbu::stream_kernel_ptr(3);
-    case K_C8: return gbu::utf8_to_utf16_kernel_ptr();
+    case K_C8: case K_C8S: return gbu::utf8_to_utf16_kernel_ptr(k == K_C8S);
     case K_V16BE: return gbu::stream_kernel_ptr(4);
     case K_L16BE: return gbu::stream_kernel_ptr(5);
-    case K_C16BE: return gbu::utf16be_to_utf8_kernel_ptr();
-    case K_C8BE: return gbu::utf8_to_utf16be_kernel_ptr();
+    case K_C16BE: case K_C16BES: return gbu::utf16be_to_utf8_kernel_ptr(k == K_C16BES);
+    case K_C8BE: case K_C8BES: return gbu::utf8_to_utf16be_kernel_ptr(k == K_C8BES);
     case K_V32: return gbu::utf32_stream_kernel_ptr(0);
     case K_L8F32: return gbu::utf32_stream_kernel_ptr(1);
     case K_L32: return gbu::utf32_stream_kernel_ptr(2);
@@ -44,18 +46,22 @@ const void *kernel_ptr(int k) {
     case K_L32F16: return gbu::utf32_stream_kernel_ptr(4);
     case K_C32T16: return gbu::utf32_to_utf16_kernel_ptr();
     case K_C16T32: return gbu::utf16_to_utf32_kernel_ptr();
-    default: return gbu::utf16_to_utf8_kernel_ptr();
+    default: return gbu::utf16_to_utf8_kernel_ptr(k == K_C16S);
   }
 }
+// the transcoders on the wide partition loop (gbu_wide.cuh); the small instances
+bool is_wide_small(int k) { return k == K_C8S || k == K_C16S || k == K_C16BES || k == K_C8BES; }
+bool is_wide(int k) { return k == K_C8 || k == K_C16 || k == K_C16BE || k == K_C8BE || is_wide_small(k); }
+int small_of(int k) { return k == K_C8 ? K_C8S : (k == K_C16 ? K_C16S : (k == K_C16BE ? K_C16BES : K_C8BES)); }
 bool is_transcoder(int k) {
-  return k == K_C8 || k == K_C16 || k == K_C16BE || k == K_C8BE || k == K_C32 || k == K_C8T32 || k == K_C32T16 ||
+  return is_wide_small(k) || k == K_C8 || k == K_C16 || k == K_C16BE || k == K_C8BE || k == K_C32 || k == K_C8T32 || k == K_C32T16 ||
          k == K_C16T32;
 }
 size_t kernel_smem(int k) {
-  if (k == K_C8) return gbu::utf8_to_utf16_smem_bytes();
-  if (k == K_C16) return gbu::utf16_to_utf8_smem_bytes();
-  if (k == K_C16BE) return gbu::utf16be_to_utf8_smem_bytes();
-  if (k == K_C8BE) return gbu::utf8_to_utf16be_smem_bytes();
+  if (k == K_C8 || k == K_C8S) return gbu::utf8_to_utf16_smem_bytes(k == K_C8S);
+  if (k == K_C16 || k == K_C16S) return gbu::utf16_to_utf8_smem_bytes(k == K_C16S);
+  if (k == K_C16BE || k == K_C16BES) return gbu::utf16be_to_utf8_smem_bytes(k == K_C16BES);
+  if (k == K_C8BE || k == K_C8BES) return gbu::utf8_to_utf16be_smem_bytes(k == K_C8BES);
   if (k == K_C32) return gbu::utf32_to_utf8_smem_bytes();
   if (k == K_C8T32) return gbu::utf8_to_utf32_smem_bytes();
   if (k == K_C32T16) return gbu::utf32_to_utf16_smem_bytes();
@@ -64,6 +70,7 @@ size_t kernel_smem(int k) {
 }
 int kernel_threads(int k) { return is_transcoder(k) ? gbu::XT : gbu::STREAM_THREADS; }
 uint32_t kernel_tile_bytes(int k) {
+  if (is_wide_small(k)) return gbu::wide_part_bytes(1);
   return is_transcoder(k) ? gbu::PART_BYTES : gbu::stream_tile_bytes();
 }
 
@@ -136,6 +143,10 @@ extern "C" gbu_ctx *gbu_create(int device, uint64_t max_units) {
   // scan states: one per transcoder partition of the largest input (UTF-32: 4 bytes per
   // unit), plus the extra partition UTF-8 inputs may use past their end
   uint64_t tiles = (4 * max_units + 64) / gbu::PART_BYTES + 4;
+  // ... or per 4 KiB partition of a small input
+  const uint64_t small_bytes = gbu::wide_small_bytes((uint64_t)c->num_sms * gbu::XBLOCKS);
+  const uint64_t span = 2 * max_units + 64 < small_bytes ? 2 * max_units + 64 : small_bytes;
+  if (span / gbu::wide_part_bytes(1) + 2 > tiles) tiles = span / gbu::wide_part_bytes(1) + 2;
   // ... and one per tile of the u64 scan of up to max_units + 1 values
   const uint64_t scan_tiles = (max_units + 1) / gbu::scan_tile_items() + 2;
   if (scan_tiles > tiles) tiles = scan_tiles;
@@ -252,8 +263,9 @@ extern "C" int gbu_launch_config(const gbu_ctx *c, int32_t *out, int n) {
   return m;
 }
 
-// Builds the launch parameters of kernel k for an input of n code units.
-static int make_params(gbu_ctx *c, int k, const void *src, uint64_t n, uint32_t unit_bytes,
+// Builds the launch parameters of kernel k for an input of n code units (k becomes its small
+// instance where that is the faster one).
+static int make_params(gbu_ctx *c, int &k, const void *src, uint64_t n, uint32_t unit_bytes,
                        bool extra_tail, gbu::Params *p) {
   if (!c) return GBU_BAD_ARGUMENT;
   if (n > c->max_units) return GBU_BAD_ARGUMENT;
@@ -264,13 +276,14 @@ static int make_params(gbu_ctx *c, int k, const void *src, uint64_t n, uint32_t 
   // the source rounded down to 16 bytes (32 for UTF-8 validation and the UTF-8 <-> UTF-16LE /
   // UTF-16BE transcoders, whose lanes read 32 bytes at a time)
   const uintptr_t a = (uintptr_t)src;
-  const uintptr_t amask = (k == K_V8 || k == K_C8 || k == K_C16 || k == K_C8BE || k == K_C16BE) ? 31 : 15;
+  const uintptr_t amask = k == K_V8 || is_wide(k) ? 31 : 15;
   p->base = (const uint8_t *)(a & ~amask);
   p->off0 = (uint32_t)(a & amask);
   p->n = n;
   p->vbytes = p->off0 + n * unit_bytes;
   // UTF-8 validation looks at the three positions past the end (a cut sequence fails there)
   const uint64_t span = n == 0 ? 0 : p->vbytes + (extra_tail ? 3 : 0);
+  if (is_wide(k) && span <= gbu::wide_small_bytes((uint64_t)c->num_sms * gbu::XBLOCKS)) k = small_of(k);
   const uint64_t tb = kernel_tile_bytes(k);
   const uint64_t ntiles = (span + tb - 1) / tb;
   if (ntiles > 0xFFFFFF00ull || (is_transcoder(k) && ntiles > c->max_states)) return GBU_BAD_ARGUMENT;
@@ -316,63 +329,69 @@ static void set_dst(gbu::Params *p, void *dst, uint64_t cap, uint32_t out_unit_b
 extern "C" int gbu_validate_utf8(gbu_ctx *c, const uint8_t *src, uint64_t n, gbu_result *result,
                                  gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_V8, src, n, 1, true, &p);
+  int k = K_V8;
+  int rc = make_params(c, k, src, n, 1, true, &p);
   if (rc != GBU_OK) return rc;
   if (!result) return GBU_BAD_ARGUMENT;
   p.result = result;
-  return launch(c, K_V8, p, stream);
+  return launch(c, k, p, stream);
 }
 
 extern "C" int gbu_validate_utf16le(gbu_ctx *c, const uint16_t *src, uint64_t n, gbu_result *result,
                                     gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_V16, src, n, 2, false, &p);
+  int k = K_V16;
+  int rc = make_params(c, k, src, n, 2, false, &p);
   if (rc != GBU_OK) return rc;
   if (!result) return GBU_BAD_ARGUMENT;
   p.result = result;
-  return launch(c, K_V16, p, stream);
+  return launch(c, k, p, stream);
 }
 
 extern "C" int gbu_utf16_length_from_utf8(gbu_ctx *c, const uint8_t *src, uint64_t n, uint64_t *len,
                                           gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_L8, src, n, 1, false, &p);
+  int k = K_L8;
+  int rc = make_params(c, k, src, n, 1, false, &p);
   if (rc != GBU_OK) return rc;
   if (!len) return GBU_BAD_ARGUMENT;
   p.len_out = len;
-  return launch(c, K_L8, p, stream);
+  return launch(c, k, p, stream);
 }
 
 extern "C" int gbu_utf8_length_from_utf16le(gbu_ctx *c, const uint16_t *src, uint64_t n, uint64_t *len,
                                             gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_L16, src, n, 2, false, &p);
+  int k = K_L16;
+  int rc = make_params(c, k, src, n, 2, false, &p);
   if (rc != GBU_OK) return rc;
   if (!len) return GBU_BAD_ARGUMENT;
   p.len_out = len;
-  return launch(c, K_L16, p, stream);
+  return launch(c, k, p, stream);
 }
 
 extern "C" int gbu_convert_utf8_to_utf16le(gbu_ctx *c, const uint8_t *src, uint64_t n, uint16_t *dst,
                                            uint64_t cap, gbu_result *result, gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_C8, src, n, 1, true, &p);
+  int k = K_C8;
+  int rc = make_params(c, k, src, n, 1, true, &p);
   if (rc != GBU_OK) return rc;
   if (!result || (cap > 0 && !dst) || ((uintptr_t)dst & 1)) return GBU_BAD_ARGUMENT;
   p.result = result;
   set_dst(&p, dst, cap, 2);
-  return launch(c, K_C8, p, stream);
+  return launch(c, k, p, stream);
 }
 
 extern "C" int gbu_convert_utf16le_to_utf8(gbu_ctx *c, const uint16_t *src, uint64_t n, uint8_t *dst,
                                            uint64_t cap, gbu_result *result, gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_C16, src, n, 2, false, &p);
+  int k = K_C16;
+  int rc = make_params(c, k, src, n, 2, false, &p);
   if (rc != GBU_OK) return rc;
   if (!result || (cap > 0 && !dst)) return GBU_BAD_ARGUMENT;
   p.result = result;
   set_dst(&p, dst, cap, 1);
-  return launch(c, K_C16, p, stream);
+  return launch(c, k, p, stream);
 }
 
 // ---- host-synchronising forms ---------------------------------------------------------------
@@ -487,95 +506,104 @@ extern "C" int gbu_per_string_loop(gbu_ctx *c, int op, const void *src, const ui
 extern "C" int gbu_validate_utf32(gbu_ctx *c, const uint32_t *src, uint64_t n, gbu_result *result,
                                   gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_V32, src, n, 4, false, &p);
+  int k = K_V32;
+  int rc = make_params(c, k, src, n, 4, false, &p);
   if (rc != GBU_OK) return rc;
   if (!result) return GBU_BAD_ARGUMENT;
   p.result = result;
-  return launch(c, K_V32, p, stream);
+  return launch(c, k, p, stream);
 }
 
 extern "C" int gbu_utf8_length_from_utf32(gbu_ctx *c, const uint32_t *src, uint64_t n, uint64_t *len,
                                           gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_L8F32, src, n, 4, false, &p);
+  int k = K_L8F32;
+  int rc = make_params(c, k, src, n, 4, false, &p);
   if (rc != GBU_OK) return rc;
   if (!len) return GBU_BAD_ARGUMENT;
   p.len_out = len;
-  return launch(c, K_L8F32, p, stream);
+  return launch(c, k, p, stream);
 }
 
 extern "C" int gbu_utf32_length_from_utf8(gbu_ctx *c, const uint8_t *src, uint64_t n, uint64_t *len,
                                           gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_L32, src, n, 1, false, &p);
+  int k = K_L32;
+  int rc = make_params(c, k, src, n, 1, false, &p);
   if (rc != GBU_OK) return rc;
   if (!len) return GBU_BAD_ARGUMENT;
   p.len_out = len;
-  return launch(c, K_L32, p, stream);
+  return launch(c, k, p, stream);
 }
 
 extern "C" int gbu_convert_utf32_to_utf8(gbu_ctx *c, const uint32_t *src, uint64_t n, uint8_t *dst,
                                          uint64_t cap, gbu_result *result, gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_C32, src, n, 4, false, &p);
+  int k = K_C32;
+  int rc = make_params(c, k, src, n, 4, false, &p);
   if (rc != GBU_OK) return rc;
   if (!result || (cap > 0 && !dst)) return GBU_BAD_ARGUMENT;
   p.result = result;
   set_dst(&p, dst, cap, 1);
-  return launch(c, K_C32, p, stream);
+  return launch(c, k, p, stream);
 }
 
 extern "C" int gbu_convert_utf8_to_utf32(gbu_ctx *c, const uint8_t *src, uint64_t n, uint32_t *dst,
                                          uint64_t cap, gbu_result *result, gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_C8T32, src, n, 1, true, &p);
+  int k = K_C8T32;
+  int rc = make_params(c, k, src, n, 1, true, &p);
   if (rc != GBU_OK) return rc;
   if (!result || (cap > 0 && !dst) || ((uintptr_t)dst & 3)) return GBU_BAD_ARGUMENT;
   p.result = result;
   set_dst(&p, dst, cap, 4);
-  return launch(c, K_C8T32, p, stream);
+  return launch(c, k, p, stream);
 }
 
 extern "C" int gbu_utf16_length_from_utf32(gbu_ctx *c, const uint32_t *src, uint64_t n, uint64_t *len,
                                            gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_L16F32, src, n, 4, false, &p);
+  int k = K_L16F32;
+  int rc = make_params(c, k, src, n, 4, false, &p);
   if (rc != GBU_OK) return rc;
   if (!len) return GBU_BAD_ARGUMENT;
   p.len_out = len;
-  return launch(c, K_L16F32, p, stream);
+  return launch(c, k, p, stream);
 }
 
 extern "C" int gbu_utf32_length_from_utf16le(gbu_ctx *c, const uint16_t *src, uint64_t n, uint64_t *len,
                                              gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_L32F16, src, n, 2, false, &p);
+  int k = K_L32F16;
+  int rc = make_params(c, k, src, n, 2, false, &p);
   if (rc != GBU_OK) return rc;
   if (!len) return GBU_BAD_ARGUMENT;
   p.len_out = len;
-  return launch(c, K_L32F16, p, stream);
+  return launch(c, k, p, stream);
 }
 
 extern "C" int gbu_convert_utf32_to_utf16le(gbu_ctx *c, const uint32_t *src, uint64_t n, uint16_t *dst,
                                             uint64_t cap, gbu_result *result, gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_C32T16, src, n, 4, false, &p);
+  int k = K_C32T16;
+  int rc = make_params(c, k, src, n, 4, false, &p);
   if (rc != GBU_OK) return rc;
   if (!result || (cap > 0 && !dst) || ((uintptr_t)dst & 1)) return GBU_BAD_ARGUMENT;
   p.result = result;
   set_dst(&p, dst, cap, 2);
-  return launch(c, K_C32T16, p, stream);
+  return launch(c, k, p, stream);
 }
 
 extern "C" int gbu_convert_utf16le_to_utf32(gbu_ctx *c, const uint16_t *src, uint64_t n, uint32_t *dst,
                                             uint64_t cap, gbu_result *result, gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_C16T32, src, n, 2, false, &p);
+  int k = K_C16T32;
+  int rc = make_params(c, k, src, n, 2, false, &p);
   if (rc != GBU_OK) return rc;
   if (!result || (cap > 0 && !dst) || ((uintptr_t)dst & 3)) return GBU_BAD_ARGUMENT;
   p.result = result;
   set_dst(&p, dst, cap, 4);
-  return launch(c, K_C16T32, p, stream);
+  return launch(c, k, p, stream);
 }
 
 // ---- UTF-16BE ----------------------------------------------------------------------------
@@ -583,43 +611,47 @@ extern "C" int gbu_convert_utf16le_to_utf32(gbu_ctx *c, const uint16_t *src, uin
 extern "C" int gbu_validate_utf16be(gbu_ctx *c, const uint16_t *src, uint64_t n, gbu_result *result,
                                     gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_V16BE, src, n, 2, false, &p);
+  int k = K_V16BE;
+  int rc = make_params(c, k, src, n, 2, false, &p);
   if (rc != GBU_OK) return rc;
   if (!result) return GBU_BAD_ARGUMENT;
   p.result = result;
-  return launch(c, K_V16BE, p, stream);
+  return launch(c, k, p, stream);
 }
 
 extern "C" int gbu_utf8_length_from_utf16be(gbu_ctx *c, const uint16_t *src, uint64_t n, uint64_t *len,
                                             gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_L16BE, src, n, 2, false, &p);
+  int k = K_L16BE;
+  int rc = make_params(c, k, src, n, 2, false, &p);
   if (rc != GBU_OK) return rc;
   if (!len) return GBU_BAD_ARGUMENT;
   p.len_out = len;
-  return launch(c, K_L16BE, p, stream);
+  return launch(c, k, p, stream);
 }
 
 extern "C" int gbu_convert_utf16be_to_utf8(gbu_ctx *c, const uint16_t *src, uint64_t n, uint8_t *dst,
                                            uint64_t cap, gbu_result *result, gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_C16BE, src, n, 2, false, &p);
+  int k = K_C16BE;
+  int rc = make_params(c, k, src, n, 2, false, &p);
   if (rc != GBU_OK) return rc;
   if (!result || (cap > 0 && !dst)) return GBU_BAD_ARGUMENT;
   p.result = result;
   set_dst(&p, dst, cap, 1);
-  return launch(c, K_C16BE, p, stream);
+  return launch(c, k, p, stream);
 }
 
 extern "C" int gbu_convert_utf8_to_utf16be(gbu_ctx *c, const uint8_t *src, uint64_t n, uint16_t *dst,
                                            uint64_t cap, gbu_result *result, gbu_stream stream) {
   gbu::Params p;
-  int rc = make_params(c, K_C8BE, src, n, 1, true, &p);
+  int k = K_C8BE;
+  int rc = make_params(c, k, src, n, 1, true, &p);
   if (rc != GBU_OK) return rc;
   if (!result || (cap > 0 && !dst) || ((uintptr_t)dst & 1)) return GBU_BAD_ARGUMENT;
   p.result = result;
   set_dst(&p, dst, cap, 2);
-  return launch(c, K_C8BE, p, stream);
+  return launch(c, k, p, stream);
 }
 
 // ---- batched forms -----------------------------------------------------------------------

@@ -768,7 +768,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_u64_kernel(const ScanParams
     }
   }
   __syncthreads();
-  if (is_last) reset_workspace(p);
+  if (is_last) reset_workspace(p, epoch);
 }
 
 // ---- host-side handles -------------------------------------------------------------------

@@ -494,9 +494,46 @@ __device__ __forceinline__ bool fold_and_finish(const Params &p, unsigned long l
   return *is_last != 0;
 }
 
-// Resets the per-launch header fields and advances the epoch (last CTA, all threads; the
+// The same in one atomic, for the read-only kernels and the wide transcoders: the header's total
+// takes, besides the CTA's units, a count of CTAs and of CTAs with an error, so that its old value
+// tells the last CTA everything (the launch's units in `units`, whether the error key is set in
+// `errors`) without another round trip to L2.  add: the CTA's units (thread 0).  Fields: CTAs from
+// bit 52, CTAs with an error from bit 40 (a grid has fewer than 4096 CTAs), units below (no buffer
+// of the device's memory gives 2^40).
+constexpr int FIN_CTAS = 52, FIN_ERRORS = 40;
+
+template <int NTH>
+__device__ __forceinline__ bool finish_packed(const Params &p, unsigned long long err_pos, unsigned long long add,
+                                              unsigned long long *red, int *is_last, unsigned long long *units,
+                                              bool *errors) {
+  constexpr int NW = NTH / 32;
+  const bool any = __syncthreads_or(err_pos != NO_ERROR);
+  if (any) {
+    err_pos = warp_min_u64(err_pos);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = err_pos;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    if (any) {
+      unsigned long long a = NO_ERROR;
+      for (int w = 0; w < NW; ++w) a = red[w] < a ? red[w] : a;
+      atomicMin(&p.ws->errkey, a);
+      __threadfence();
+    }
+    const unsigned long long one = 1ull << FIN_CTAS | (any ? 1ull << FIN_ERRORS : 0ull) | add;
+    const unsigned long long now = atomicAdd(&p.ws->total, one) + one;
+    *is_last = (now >> FIN_CTAS) == gridDim.x;
+    *units = now & ((1ull << FIN_ERRORS) - 1);
+    *errors = (now >> FIN_ERRORS & ((1ull << (FIN_CTAS - FIN_ERRORS)) - 1)) != 0;
+    if (*is_last) __threadfence();
+  }
+  __syncthreads();
+  return *is_last != 0;
+}
+
+// Resets the per-launch header fields and advances the epoch (the launch's; last CTA, all threads; the
 // whole CTA clears the scan states when the epoch wraps).
-__device__ __forceinline__ void reset_workspace(const Params &p) {
+__device__ __forceinline__ void reset_workspace(const Params &p, uint32_t epoch) {
   __shared__ uint32_t wrap;
   if (threadIdx.x == 0) {
     WsHeader *ws = p.ws;
@@ -506,7 +543,7 @@ __device__ __forceinline__ void reset_workspace(const Params &p) {
     ws->total = 0;
     ws->status = 0;
     ws->stop_tile = 0xFFFFFFFFu;
-    const uint32_t e = ws->epoch + 1;
+    const uint32_t e = epoch + 1;
     wrap = e > ST_EPOCH_MASK;
     ws->epoch = wrap ? 1u : e;
   }

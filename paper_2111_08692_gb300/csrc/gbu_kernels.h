@@ -12,16 +12,17 @@ const void *stream_kernel_ptr(int mode);
 uint32_t stream_tile_bytes();
 
 // transcoders (dynamic shared memory of the given size; above 48 KB it needs the
-// cudaFuncAttributeMaxDynamicSharedMemorySize opt-in before the first launch)
-const void *utf8_to_utf16_kernel_ptr();
-const void *utf16_to_utf8_kernel_ptr();
-size_t utf8_to_utf16_smem_bytes();
-size_t utf16_to_utf8_smem_bytes();
+// cudaFuncAttributeMaxDynamicSharedMemorySize opt-in before the first launch); small: the instance
+// on 4 KiB partitions
+const void *utf8_to_utf16_kernel_ptr(bool small);
+const void *utf16_to_utf8_kernel_ptr(bool small);
+size_t utf8_to_utf16_smem_bytes(bool small);
+size_t utf16_to_utf8_smem_bytes(bool small);
 // the transcoders between UTF-8 and UTF-16BE (same launch shape as the UTF-16LE ones)
-const void *utf16be_to_utf8_kernel_ptr();
-size_t utf16be_to_utf8_smem_bytes();
-const void *utf8_to_utf16be_kernel_ptr();
-size_t utf8_to_utf16be_smem_bytes();
+const void *utf16be_to_utf8_kernel_ptr(bool small);
+size_t utf16be_to_utf8_smem_bytes(bool small);
+const void *utf8_to_utf16be_kernel_ptr(bool small);
+size_t utf8_to_utf16be_smem_bytes(bool small);
 // UTF-32: read-only kernel (mode 0 validate_utf32, 1 utf8_length_from_utf32,
 // 2 utf32_length_from_utf8, 3 utf16_length_from_utf32, 4 utf32_length_from_utf16le) and the
 // transcoders between UTF-32 and UTF-8 / UTF-16LE

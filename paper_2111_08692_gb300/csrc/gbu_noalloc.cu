@@ -62,11 +62,11 @@ int setup_device(DeviceSetup &s, int device) {
     return GBU_CUDA_ERROR;
   }
   int sms = 0, bps = 0;
-  const size_t smem = gbu::utf8_to_utf16_smem_bytes();
-  if (cudaFuncSetAttribute(gbu::utf8_to_utf16_kernel_ptr(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const size_t smem = gbu::utf8_to_utf16_smem_bytes(false);
+  if (cudaFuncSetAttribute(gbu::utf8_to_utf16_kernel_ptr(false), cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)smem) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, gbu::utf8_to_utf16_kernel_ptr(), gbu::XT, smem) !=
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, gbu::utf8_to_utf16_kernel_ptr(false), gbu::XT, smem) !=
           cudaSuccess ||
       sms < 1 || bps < 1) {
     cudaGetLastError();
@@ -146,8 +146,8 @@ extern "C" int gbu_convert_utf8_to_utf16le_noalloc(const uint8_t *src, uint64_t 
   if (p.ntiles < grid) grid = p.ntiles;
   if (grid < 1) grid = 1;
   void *args[] = {(void *)&p};
-  if (cudaLaunchKernel(gbu::utf8_to_utf16_kernel_ptr(), dim3(grid), dim3(gbu::XT), args,
-                       gbu::utf8_to_utf16_smem_bytes(), (cudaStream_t)stream) != cudaSuccess) {
+  if (cudaLaunchKernel(gbu::utf8_to_utf16_kernel_ptr(false), dim3(grid), dim3(gbu::XT), args,
+                       gbu::utf8_to_utf16_smem_bytes(false), (cudaStream_t)stream) != cudaSuccess) {
     cudaGetLastError();
     return GBU_CUDA_ERROR;
   }

@@ -40,6 +40,14 @@ __host__ __device__ constexpr int stream_min_blocks() {
   return (base_mode<MODE>() == S_L16 || base_mode<MODE>() == S_L8) ? 4 : 3;
 }
 
+// What a read-only launch has changed in the header (last CTA, thread 0); it uses no scan states, so
+// their epoch stays.
+__device__ __forceinline__ void reset_read_only(WsHeader *ws) {
+  ws->total = 0;
+  ws->errkey = NO_ERROR;
+  ws->stop_tile = 0xFFFFFFFFu;
+}
+
 template <int KMODE>
 __global__ void __launch_bounds__(STREAM_THREADS, stream_min_blocks<KMODE>()) stream_kernel(const Params p) {
   constexpr int MODE = base_mode<KMODE>();
@@ -206,23 +214,31 @@ __global__ void __launch_bounds__(STREAM_THREADS, stream_min_blocks<KMODE>()) st
     if (early && stop_after_tile(wt, snap)) break;
   }
 
-  const bool want_err = MODE == S_V16;
-  if (!fold_and_finish<STREAM_THREADS>(p, want_err ? err_pos : total, want_err, red, &is_last)) return;
+  unsigned long long cta = 0;
+  if (MODE == S_L16 || MODE == S_L8) {
+    total = warp_sum_u64(total);
+    if (lane == 0) red[warp] = total;
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int w = 0; w < ST_WARPS; ++w) cta += red[w];
+  }
+  unsigned long long tot;
+  bool errors;
+  if (!finish_packed<STREAM_THREADS>(p, err_pos, cta, red, &is_last, &tot, &errors)) return;
   if (threadIdx.x == 0) {
-    const unsigned long long key = *(volatile unsigned long long *)&p.ws->errkey;
-    const unsigned long long tot = *(volatile unsigned long long *)&p.ws->total;
     if (MODE == S_L16 || MODE == S_L8) {
       *p.len_out = tot;
-    } else if (key == NO_ERROR) {
+    } else if (!errors) {
       write_result(p.result, GBU_OK, p.n);
     } else {
+      const unsigned long long key = *(volatile unsigned long long *)&p.ws->errkey;
       uint64_t off;
       resolve_utf16_error<BE>(reinterpret_cast<const uint16_t *>(p.base + p.off0), p.n,
                               ((long long)key - (long long)p.off0) / 2, &off);
       write_result(p.result, GBU_SURROGATE, off);
     }
+    reset_read_only(p.ws);
   }
-  reset_workspace(p);
 }
 
 // UTF-8 validation: a warp streams 4 KiB warp tiles, four regions of 1 KiB, a lane 32 consecutive
@@ -316,19 +332,21 @@ __global__ void __launch_bounds__(STREAM_THREADS, 3) validate8_kernel(const Para
       if ((it & 7u) == 1u) known = __shfl_sync(0xffffffffu, snap, 0);
     }
   }
-  if (!fold_and_finish<STREAM_THREADS>(p, err_pos, true, red, &is_last)) return;
+  unsigned long long tot;
+  bool errors;
+  if (!finish_packed<STREAM_THREADS>(p, err_pos, 0, red, &is_last, &tot, &errors)) return;
   if (threadIdx.x == 0) {
-    const unsigned long long key = *(volatile unsigned long long *)&p.ws->errkey;
-    if (key == NO_ERROR) {
+    if (!errors) {
       write_result(p.result, GBU_OK, p.n);
     } else {
+      const unsigned long long key = *(volatile unsigned long long *)&p.ws->errkey;
       int32_t kind;
       uint64_t off;
       resolve_utf8_error(p.base + p.off0, p.n, (long long)key - (long long)p.off0, &kind, &off);
       write_result(p.result, kind, off);
     }
+    reset_read_only(p.ws);
   }
-  reset_workspace(p);
 }
 
 const void *stream_kernel_ptr(int mode) {

@@ -9,10 +9,11 @@
 
 namespace gbu {
 
+template <int R>
 __global__ void __launch_bounds__(XT, XBLOCKS) utf16_to_utf8_kernel(const Params p) {
   extern __shared__ __align__(128) unsigned char smem_raw[];  // sizeof(WSmem), set at launch
-  WSmem<Utf16ToUtf8Wide> &sm = *reinterpret_cast<WSmem<Utf16ToUtf8Wide> *>(smem_raw);
-  wtranscode<Utf16ToUtf8Wide>(p, sm, [&](uint32_t status, unsigned long long key, unsigned long long tot) {
+  WSmem<Utf16ToUtf8Wide, R> &sm = *reinterpret_cast<WSmem<Utf16ToUtf8Wide, R> *>(smem_raw);
+  wtranscode<Utf16ToUtf8Wide, R>(p, sm, [&](uint32_t status, unsigned long long key, unsigned long long tot) {
     if (status) {
       write_result(p.result, GBU_TIMEOUT, 0);
     } else if (key != NO_ERROR) {
@@ -47,8 +48,12 @@ __global__ void __launch_bounds__(XT, XBLOCKS) utf16_to_utf8_segments_kernel(con
   });
 }
 
-const void *utf16_to_utf8_kernel_ptr() { return (const void *)utf16_to_utf8_kernel; }
-size_t utf16_to_utf8_smem_bytes() { return sizeof(WSmem<Utf16ToUtf8Wide>); }
+const void *utf16_to_utf8_kernel_ptr(bool small) {
+  return small ? (const void *)utf16_to_utf8_kernel<1> : (const void *)utf16_to_utf8_kernel<WROUNDS>;
+}
+size_t utf16_to_utf8_smem_bytes(bool small) {
+  return small ? sizeof(WSmem<Utf16ToUtf8Wide, 1>) : sizeof(WSmem<Utf16ToUtf8Wide, WROUNDS>);
+}
 size_t utf16_to_utf8_segments_smem_bytes() { return sizeof(XSmem<Utf16ToUtf8>); }
 
 const void *utf16_to_utf8_segments_kernel_ptr() { return (const void *)utf16_to_utf8_segments_kernel; }

@@ -76,10 +76,11 @@ struct Utf8ToUtf16BEWide : Utf8ToUtf16Wide {
   }
 };
 
+template <int R>
 __global__ void __launch_bounds__(XT, XBLOCKS) utf16be_to_utf8_kernel(const Params p) {
   extern __shared__ __align__(128) unsigned char smem_raw[];  // sizeof(WSmem), set at launch
-  WSmem<Utf16BEToUtf8Wide> &sm = *reinterpret_cast<WSmem<Utf16BEToUtf8Wide> *>(smem_raw);
-  wtranscode<Utf16BEToUtf8Wide>(p, sm, [&](uint32_t status, unsigned long long key, unsigned long long tot) {
+  WSmem<Utf16BEToUtf8Wide, R> &sm = *reinterpret_cast<WSmem<Utf16BEToUtf8Wide, R> *>(smem_raw);
+  wtranscode<Utf16BEToUtf8Wide, R>(p, sm, [&](uint32_t status, unsigned long long key, unsigned long long tot) {
     if (status) {
       write_result(p.result, GBU_TIMEOUT, 0);
     } else if (key != NO_ERROR) {
@@ -93,10 +94,11 @@ __global__ void __launch_bounds__(XT, XBLOCKS) utf16be_to_utf8_kernel(const Para
   });
 }
 
+template <int R>
 __global__ void __launch_bounds__(XT, XBLOCKS) utf8_to_utf16be_kernel(const Params p) {
   extern __shared__ __align__(128) unsigned char smem_raw[];  // sizeof(WSmem), set at launch
-  WSmem<Utf8ToUtf16BEWide> &sm = *reinterpret_cast<WSmem<Utf8ToUtf16BEWide> *>(smem_raw);
-  wtranscode<Utf8ToUtf16BEWide>(p, sm, [&](uint32_t status, unsigned long long key, unsigned long long tot) {
+  WSmem<Utf8ToUtf16BEWide, R> &sm = *reinterpret_cast<WSmem<Utf8ToUtf16BEWide, R> *>(smem_raw);
+  wtranscode<Utf8ToUtf16BEWide, R>(p, sm, [&](uint32_t status, unsigned long long key, unsigned long long tot) {
     if (status) {
       write_result(p.result, GBU_TIMEOUT, 0);
     } else if (key != NO_ERROR) {
@@ -110,9 +112,17 @@ __global__ void __launch_bounds__(XT, XBLOCKS) utf8_to_utf16be_kernel(const Para
   });
 }
 
-const void *utf16be_to_utf8_kernel_ptr() { return (const void *)utf16be_to_utf8_kernel; }
-size_t utf16be_to_utf8_smem_bytes() { return sizeof(WSmem<Utf16BEToUtf8Wide>); }
-const void *utf8_to_utf16be_kernel_ptr() { return (const void *)utf8_to_utf16be_kernel; }
-size_t utf8_to_utf16be_smem_bytes() { return sizeof(WSmem<Utf8ToUtf16BEWide>); }
+const void *utf16be_to_utf8_kernel_ptr(bool small) {
+  return small ? (const void *)utf16be_to_utf8_kernel<1> : (const void *)utf16be_to_utf8_kernel<WROUNDS>;
+}
+size_t utf16be_to_utf8_smem_bytes(bool small) {
+  return small ? sizeof(WSmem<Utf16BEToUtf8Wide, 1>) : sizeof(WSmem<Utf16BEToUtf8Wide, WROUNDS>);
+}
+const void *utf8_to_utf16be_kernel_ptr(bool small) {
+  return small ? (const void *)utf8_to_utf16be_kernel<1> : (const void *)utf8_to_utf16be_kernel<WROUNDS>;
+}
+size_t utf8_to_utf16be_smem_bytes(bool small) {
+  return small ? sizeof(WSmem<Utf8ToUtf16BEWide, 1>) : sizeof(WSmem<Utf8ToUtf16BEWide, WROUNDS>);
+}
 
 }  // namespace gbu

@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(STREAM_THREADS) utf32_stream_kernel(const Para
       write_result(p.result, kind, off);
     }
   }
-  reset_workspace(p);
+  reset_workspace(p, p.ws->epoch);
 }
 
 // ---- UTF-32 -> UTF-8 codec ------------------------------------------------------------------

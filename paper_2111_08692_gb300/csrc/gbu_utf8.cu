@@ -9,10 +9,11 @@
 
 namespace gbu {
 
+template <int R>
 __global__ void __launch_bounds__(XT, XBLOCKS) utf8_to_utf16_kernel(const Params p) {
   extern __shared__ __align__(128) unsigned char smem_raw[];  // sizeof(WSmem), set at launch
-  WSmem<Utf8ToUtf16Wide> &sm = *reinterpret_cast<WSmem<Utf8ToUtf16Wide> *>(smem_raw);
-  wtranscode<Utf8ToUtf16Wide>(p, sm, [&](uint32_t status, unsigned long long key, unsigned long long tot) {
+  WSmem<Utf8ToUtf16Wide, R> &sm = *reinterpret_cast<WSmem<Utf8ToUtf16Wide, R> *>(smem_raw);
+  wtranscode<Utf8ToUtf16Wide, R>(p, sm, [&](uint32_t status, unsigned long long key, unsigned long long tot) {
     if (status) {
       write_result(p.result, GBU_TIMEOUT, 0);
     } else if (key != NO_ERROR) {
@@ -47,8 +48,12 @@ __global__ void __launch_bounds__(XT, XBLOCKS) utf8_to_utf16_segments_kernel(con
   });
 }
 
-const void *utf8_to_utf16_kernel_ptr() { return (const void *)utf8_to_utf16_kernel; }
-size_t utf8_to_utf16_smem_bytes() { return sizeof(WSmem<Utf8ToUtf16Wide>); }
+const void *utf8_to_utf16_kernel_ptr(bool small) {
+  return small ? (const void *)utf8_to_utf16_kernel<1> : (const void *)utf8_to_utf16_kernel<WROUNDS>;
+}
+size_t utf8_to_utf16_smem_bytes(bool small) {
+  return small ? sizeof(WSmem<Utf8ToUtf16Wide, 1>) : sizeof(WSmem<Utf8ToUtf16Wide, WROUNDS>);
+}
 size_t utf8_to_utf16_segments_smem_bytes() { return sizeof(XSmem<Utf8ToUtf16>); }
 
 const void *utf8_to_utf16_segments_kernel_ptr() { return (const void *)utf8_to_utf16_segments_kernel; }

@@ -1,7 +1,8 @@
 // gbu_wide.cuh -- the partition loop of the single-buffer UTF-8 <-> UTF-16LE transcoders, with
 // 32 input bytes per lane and 1 KiB warp regions.
 //
-// The loop has the shape of gbu_xcode.cuh's: a CTA of XT threads claims 16 KiB partitions from
+// The loop has the shape of gbu_xcode.cuh's: a CTA of XT threads claims partitions of R x 4 KiB
+// (16 KiB, or 4 KiB for small inputs: see WIDE_SMALL_BYTES) from
 // a ticket counter, counts the output of the NEXT partition (a read from HBM) and publishes
 // that aggregate before it takes the CURRENT partition's output offset from the CTA-wide
 // decoupled look-back, then converts the current partition (a re-read, normally from L2)
@@ -12,7 +13,7 @@
 //   * a lane owns 32 consecutive bytes of its region, read by one 256-bit load; the words just
 //     before and after them come from the adjacent lanes, or from the previous region's lane 31
 //     and the next region's lane 0;
-//   * warp w owns the w-th 4 KiB slice of the partition, four regions of 1 KiB;
+//   * warp w owns the w-th slice of the partition, R regions of 1 KiB;
 //   * the count pass keeps, per region, every lane's exclusive output offset and the region's
 //     total and codec flags, and per slice its total; a warp finds its regions' offsets from
 //     the slice totals of the warps before it and a running sum over its own regions.
@@ -46,21 +47,30 @@ namespace gbu {
 
 constexpr uint32_t WLANE = 32;                        // input bytes per lane per region
 constexpr uint32_t WREGION = 32 * WLANE;              // 1 KiB per warp region
-constexpr int WROUNDS = (int)(SLICE_BYTES / WREGION); // regions per warp slice
-constexpr int WREGIONS = WROUNDS * XWARPS;            // regions per partition
+constexpr int WROUNDS = (int)(SLICE_BYTES / WREGION);  // regions per warp slice (R) of a 16 KiB partition
 static_assert(SLICE_BYTES == WREGION * WROUNDS, "a slice is whole regions");
-static_assert(WROUNDS % 2 == 0, "the count pass scans two regions at a time");
+// Bytes of a partition with R regions per slice.
+__host__ __device__ constexpr uint32_t wide_part_bytes(int R) { return (uint32_t)(R * XWARPS) * WREGION; }
+// Small inputs run on partitions of one region per warp (4 KiB): four times as many CTAs share the
+// work, and a warp converts one region instead of four in a row.  The line lies at one and a half
+// such partitions per resident CTA (7.5 MB on 152 SMs); past it the fixed work per partition
+// counts.  Mixed text, 4 KiB / 16 KiB partitions, us per launch (GB300), 8 -> 16: 4 KB 7.7 / 19.5,
+// 1 MiB 10.1 / 23.7, 4 MiB 15.6 / 24.0, 6 MiB 21.3 / 25.6, 16 MiB 36.0 / 39.2; 16 -> 8: 4 KB 10.5 /
+// 17.9, 1 MiB 12.7 / 21.2, 4 MiB 18.9 / 22.5, 8 MiB 28.2 / 28.5, 16 MiB 44.7 / 42.3.
+__host__ __device__ constexpr uint64_t wide_small_bytes(uint64_t ctas) { return ctas * wide_part_bytes(1) * 3 / 2; }
 
+template <int R>
 struct __align__(16) WideCounts {
-  uint16_t lane_off[WREGIONS][32];  // each lane's exclusive offset inside its region
-  uint32_t rinfo[WREGIONS];         // region total (bits 0-15) | codec flags << 16
-  uint32_t slice[XWARPS];           // slice total (bits 0-30) | 1 << 31 for an all-ASCII slice inside the buffer
+  static constexpr int REGIONS = R * XWARPS;
+  uint16_t lane_off[REGIONS][32];  // each lane's exclusive offset inside its region
+  uint32_t rinfo[REGIONS];         // region total (bits 0-15) | codec flags << 16
+  uint32_t slice[XWARPS];          // slice total (bits 0-30) | 1 << 31 for an all-ASCII slice inside the buffer
 };
 
-template <class Codec>
+template <class Codec, int R>
 struct __align__(128) WSmem {
   typename Codec::Out staging[XWARPS][2][Codec::WSTAGE];
-  WideCounts counts[2];
+  WideCounts<R> counts[2];
   LookbackSmem<XT> lb;
   unsigned long long red[XWARPS];
   uint32_t ticket;
@@ -89,29 +99,38 @@ __device__ __forceinline__ void load32(const Params &p, long long c, bool inside
 }
 
 // Virtual position of lane `lane`'s 32 bytes in region r of warp w's slice of partition part.
+template <int R>
 __device__ __forceinline__ long long wchunk_pos(uint32_t part, int w, int r, int lane) {
-  return (long long)part * PART_BYTES + (long long)w * SLICE_BYTES + (long long)r * WREGION +
+  return (long long)part * wide_part_bytes(R) + (long long)w * (R * WREGION) + (long long)r * WREGION +
          (long long)lane * WLANE;
+}
+
+// Whether partition `part` lies inside the buffer with a word to spare at each end.
+template <int R>
+__device__ __forceinline__ bool wpart_inside(const Params &p, uint32_t part) {
+  const long long p0 = (long long)part * wide_part_bytes(R);
+  return p0 - 4 >= (long long)p.off0 && p0 + (long long)wide_part_bytes(R) + 4 <= (long long)p.vbytes;
 }
 
 // Counts partition `part` into pc (all threads; the caller puts a barrier after it).  INSIDE:
 // the partition lies inside the buffer with a word to spare at each end.
-template <class Codec, bool INSIDE>
-__device__ __forceinline__ void wcount_partition(const Params &p, uint32_t part, WideCounts &pc) {
+template <class Codec, int R, bool INSIDE>
+__device__ __forceinline__ void wcount_partition(const Params &p, uint32_t part, WideCounts<R> &pc) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const long long s0 = wchunk_pos(part, warp, 0, 0);
+  constexpr uint32_t SLICE = R * WREGION;
+  const long long s0 = wchunk_pos<R>(part, warp, 0, 0);
   const long long lo = p.off0, hi = (long long)p.vbytes;
-  const bool inside = INSIDE || (s0 >= lo && s0 + (long long)SLICE_BYTES <= hi);
+  const bool inside = INSIDE || (s0 >= lo && s0 + (long long)SLICE <= hi);
   // the slice is read again by its conversion one partition later: keep it in L2
   const uint64_t keep = l2_policy_keep();
-  uint32_t v[WROUNDS][8];
+  uint32_t v[R][8];
 #pragma unroll
-  for (int r = 0; r < WROUNDS; ++r) load32(p, s0 + (long long)r * WREGION + WLANE * lane, inside, keep, v[r]);
+  for (int r = 0; r < R; ++r) load32(p, s0 + (long long)r * WREGION + WLANE * lane, inside, keep, v[r]);
   bool slice_ascii = false;
   if (INSIDE) {
     uint32_t any = 0;
 #pragma unroll
-    for (int r = 0; r < WROUNDS; ++r)
+    for (int r = 0; r < R; ++r)
 #pragma unroll
       for (int k = 0; k < 8; ++k) any |= v[r][k];
     slice_ascii = __all_sync(0xffffffffu, (any & Codec::ASCII_MASK) == 0);
@@ -120,15 +139,16 @@ __device__ __forceinline__ void wcount_partition(const Params &p, uint32_t part,
   if (slice_ascii) {
     // every lane gives LANE_UNITS units: no scan needed
 #pragma unroll
-    for (int r = 0; r < WROUNDS; ++r) pc.lane_off[warp * WROUNDS + r][lane] = (uint16_t)(lane * Codec::LANE_UNITS);
-    if (lane < WROUNDS) pc.rinfo[warp * WROUNDS + lane] = Codec::WREGION_UNITS;
-    stot = WROUNDS * Codec::WREGION_UNITS;
+    for (int r = 0; r < R; ++r) pc.lane_off[warp * R + r][lane] = (uint16_t)(lane * Codec::LANE_UNITS);
+    if (lane < R) pc.rinfo[warp * R + lane] = Codec::WREGION_UNITS;
+    stot = R * Codec::WREGION_UNITS;
   } else {
 #pragma unroll
-    for (int r = 0; r < WROUNDS; r += 2) {
+    for (int r = 0; r < R; r += 2) {
       uint32_t a[2], f[2];
+      if (r + 1 >= R) a[1] = f[1] = 0u;
 #pragma unroll
-      for (int q = 0; q < 2; ++q) {
+      for (int q = 0; q < (r + 1 < R ? 2 : 1); ++q) {
         const long long c = s0 + (long long)(r + q) * WREGION + WLANE * lane;
         const bool edge = !inside && (c < lo || c + (long long)WLANE > hi);
         a[q] = Codec::wcount(p, v[r + q], c, edge, f[q]);
@@ -148,13 +168,14 @@ __device__ __forceinline__ void wcount_partition(const Params &p, uint32_t part,
         }
       }
       const uint32_t ex = incl - x;
-      const int ri = warp * WROUNDS + r;
+      const int ri = warp * R + r;
       pc.lane_off[ri][lane] = (uint16_t)(ex & 0xFFFFu);
-      pc.lane_off[ri + 1][lane] = (uint16_t)(ex >> 16);
-      const uint32_t fr0 = __reduce_or_sync(0xffffffffu, f[0]), fr1 = __reduce_or_sync(0xffffffffu, f[1]);
+      if (r + 1 < R) pc.lane_off[ri + 1][lane] = (uint16_t)(ex >> 16);
+      const uint32_t fr0 = __reduce_or_sync(0xffffffffu, f[0]);
+      const uint32_t fr1 = r + 1 < R ? __reduce_or_sync(0xffffffffu, f[1]) : 0u;
       if (lane == 31) {
         pc.rinfo[ri] = (incl & 0xFFFFu) | (fr0 << 16);
-        pc.rinfo[ri + 1] = (incl >> 16) | (fr1 << 16);
+        if (r + 1 < R) pc.rinfo[ri + 1] = (incl >> 16) | (fr1 << 16);
       }
       stot += (incl & 0xFFFFu) + (incl >> 16);  // meaningful in lane 31
     }
@@ -164,18 +185,19 @@ __device__ __forceinline__ void wcount_partition(const Params &p, uint32_t part,
 
 // Step 3 for partition `part` (all threads; each warp on its slice): transcodes the
 // partition, whose output starts at unit S0, with the counts of its count pass in pc.
-template <class Codec, bool INSIDE>
-__device__ __forceinline__ void wconvert_partition(const Params &p, uint32_t part, const WideCounts &pc, uint64_t S0,
-                                                   WSmem<Codec> &sm, uint32_t &use, unsigned long long &err_pos) {
+template <class Codec, int R, bool INSIDE>
+__device__ __forceinline__ void wconvert_partition(const Params &p, uint32_t part, const WideCounts<R> &pc,
+                                                   uint64_t S0, WSmem<Codec, R> &sm, uint32_t &use, unsigned long long &err_pos) {
   using Out = typename Codec::Out;
   constexpr uint32_t V = 16 / sizeof(Out);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long lo = p.off0, hi = (long long)p.vbytes;
-  const long long s0 = wchunk_pos(part, warp, 0, 0);
-  const bool slice_inside = INSIDE || (s0 - 4 >= lo && s0 + (long long)SLICE_BYTES + 4 <= hi);
+  constexpr uint32_t SLICE = R * WREGION;
+  const long long s0 = wchunk_pos<R>(part, warp, 0, 0);
+  const bool slice_inside = INSIDE || (s0 - 4 >= lo && s0 + (long long)SLICE + 4 <= hi);
   const uint32_t before = slice_inside ? ldg_word(p.base + s0 - 4) : load_word_checked(p, s0 - 4);
   const uint32_t after =
-      slice_inside ? ldg_word(p.base + s0 + SLICE_BYTES) : load_word_checked(p, s0 + SLICE_BYTES);
+      slice_inside ? ldg_word(p.base + s0 + SLICE) : load_word_checked(p, s0 + SLICE);
   // the slice's first output unit inside the partition: the totals of the slices before it
   uint32_t sbase = 0;
 #pragma unroll
@@ -192,15 +214,15 @@ __device__ __forceinline__ void wconvert_partition(const Params &p, uint32_t par
   const uint64_t last_use = l2_policy_last_use();
   const uint8_t *const src = p.base + s0 + WLANE * lane;  // the lane's 32 bytes of region 0
   if (INSIDE && (sinfo >> 31) && ((uint32_t)D0 & (Codec::WDIRECT_ALIGN - 1)) == 0 &&
-      room0 >= (uint32_t)WROUNDS * Codec::WREGION_UNITS) {
+      room0 >= (uint32_t)R * Codec::WREGION_UNITS) {
     // an all-ASCII slice whose output is aligned and fits: every region goes straight to
     // global memory; only the word before the slice can hold a leading byte that wants
     // continuation bytes in it
-    uint32_t w[WROUNDS][8];
+    uint32_t w[R][8];
 #pragma unroll
-    for (int r = 0; r < WROUNDS; ++r) ldg32_hint(src + r * WREGION, last_use, w[r]);
+    for (int r = 0; r < R; ++r) ldg32_hint(src + r * WREGION, last_use, w[r]);
 #pragma unroll
-    for (int r = 0; r < WROUNDS; ++r)
+    for (int r = 0; r < R; ++r)
       Codec::wascii_direct(dslice + r * Codec::WREGION_UNITS, w[r], r == 0 ? before : 0u,
                            s0 + (long long)r * WREGION + WLANE * lane, err_pos);
     return;
@@ -208,7 +230,7 @@ __device__ __forceinline__ void wconvert_partition(const Params &p, uint32_t par
   uint32_t prev_last = before;  // last word of the previous region (lane 31's), for lane 0
   uint32_t off = 0;             // the region's first unit inside the slice's output
 #pragma unroll 1
-  for (int r = 0; r < WROUNDS; ++r) {
+  for (int r = 0; r < R; ++r) {
     const long long c = s0 + (long long)r * WREGION + WLANE * lane;
     const bool edge = !INSIDE && (c < lo || c + (long long)WLANE > hi);
     // the lane's 32 bytes (other warps cover the L2 latency; a load kept a region ahead would
@@ -217,7 +239,7 @@ __device__ __forceinline__ void wconvert_partition(const Params &p, uint32_t par
     uint32_t v[8];
     load32(p, c, slice_inside, last_use, v);
     uint32_t next_first = after;
-    if (lane == 31 && r + 1 < WROUNDS)
+    if (lane == 31 && r + 1 < R)
       next_first = slice_inside ? ldg_word(p.base + c + WLANE) : load_word_checked(p, c + WLANE);
     uint32_t prev = __shfl_up_sync(0xffffffffu, v[7], 1);
     uint32_t next = __shfl_down_sync(0xffffffffu, v[0], 1);
@@ -225,7 +247,7 @@ __device__ __forceinline__ void wconvert_partition(const Params &p, uint32_t par
     if (lane == 31) next = next_first;
     prev_last = __shfl_sync(0xffffffffu, v[7], 31);
 
-    const int ri = warp * WROUNDS + r;
+    const int ri = warp * R + r;
     const uint32_t info = pc.rinfo[ri];
     const uint32_t rtot = info & 0xFFFFu, rflags = info >> 16;
     const uint32_t dlo = (uint32_t)D0 + off;  // low bits of the region's destination unit
@@ -252,21 +274,22 @@ __device__ __forceinline__ void wconvert_partition(const Params &p, uint32_t par
   }
 }
 
-template <class Codec>
-__device__ __forceinline__ void wcount_part(const Params &p, uint32_t part, WideCounts &pc) {
-  if (part_inside(p, part)) wcount_partition<Codec, true>(p, part, pc);
-  else wcount_partition<Codec, false>(p, part, pc);
+template <class Codec, int R>
+__device__ __forceinline__ void wcount_part(const Params &p, uint32_t part, WideCounts<R> &pc) {
+  if (wpart_inside<R>(p, part)) wcount_partition<Codec, R, true>(p, part, pc);
+  else wcount_partition<Codec, R, false>(p, part, pc);
 }
 
-template <class Codec>
-__device__ __forceinline__ void wconvert_part(const Params &p, uint32_t part, const WideCounts &pc, uint64_t S0,
-                                              WSmem<Codec> &sm, uint32_t &use, unsigned long long &err_pos) {
-  if (part_inside(p, part)) wconvert_partition<Codec, true>(p, part, pc, S0, sm, use, err_pos);
-  else wconvert_partition<Codec, false>(p, part, pc, S0, sm, use, err_pos);
+template <class Codec, int R>
+__device__ __forceinline__ void wconvert_part(const Params &p, uint32_t part, const WideCounts<R> &pc, uint64_t S0,
+                                              WSmem<Codec, R> &sm, uint32_t &use, unsigned long long &err_pos) {
+  if (wpart_inside<R>(p, part)) wconvert_partition<Codec, R, true>(p, part, pc, S0, sm, use, err_pos);
+  else wconvert_partition<Codec, R, false>(p, part, pc, S0, sm, use, err_pos);
 }
 
 // The partition's total output (after the barrier that follows its count pass).
-__device__ __forceinline__ uint32_t wpart_total(const WideCounts &pc) {
+template <int R>
+__device__ __forceinline__ uint32_t wpart_total(const WideCounts<R> &pc) {
   uint32_t t = 0;
 #pragma unroll
   for (int w = 0; w < XWARPS; ++w) t += pc.slice[w] & 0x7FFFFFFFu;
@@ -275,8 +298,8 @@ __device__ __forceinline__ uint32_t wpart_total(const WideCounts &pc) {
 
 // The whole transcoder kernel body.  finalize(status, key, total) runs in thread 0 of the
 // last CTA and writes the result.
-template <class Codec, class Final>
-__device__ __forceinline__ void wtranscode(const Params &p, WSmem<Codec> &sm, Final finalize) {
+template <class Codec, int R, class Final>
+__device__ __forceinline__ void wtranscode(const Params &p, WSmem<Codec, R> &sm, Final finalize) {
   const int tid = threadIdx.x, lane = tid & 31;
   const uint32_t epoch = p.ws->epoch;
   unsigned long long err_pos = NO_ERROR;
@@ -287,25 +310,25 @@ __device__ __forceinline__ void wtranscode(const Params &p, WSmem<Codec> &sm, Fi
   __syncthreads();
   uint32_t cur = sm.ticket;
   uint32_t cur_total = 0;
+  unsigned long long all_units = 0;  // of the partitions this CTA counted
   if (cur < p.ntiles) {
-    wcount_part<Codec>(p, cur, sm.counts[cb]);
+    wcount_part<Codec, R>(p, cur, sm.counts[cb]);
     __syncthreads();
     cur_total = wpart_total(sm.counts[cb]);
-    if (tid == 0) {
-      publish_aggregate(p, cur, cur_total, epoch);
-      atomicAdd(&p.ws->total, (unsigned long long)cur_total);
-    }
+    all_units = cur_total;
+    if (tid == 0) publish_aggregate(p, cur, cur_total, epoch);
   }
-  // Early exit: output past the first error is unspecified, so a partition that starts past
-  // a chunk some thread already flagged (the error key, published at once) is counted and
-  // chained as usual -- later partitions still need its aggregate -- but not converted.  The
-  // first error lies at most 31 bytes past the smallest flagged chunk, so it is always
-  // converted up to its start.
+  // Early exit: output past the first error is unspecified, so a CTA stops at a partition that
+  // starts past a chunk some thread already flagged (the error key, published at once): later
+  // partitions, if anyone still works on them, need no more than the aggregates it has published
+  // for that partition and the next.  The first error lies at most 31 bytes past the smallest
+  // flagged chunk, so it is always converted up to its start.
   unsigned long long published = NO_ERROR;
   while (cur < p.ntiles) {
     // claim and count the next partition, so that its aggregate is out a partition early
     if (tid == 0) {
-      sm.ticket = atomicAdd(&p.ws->ticket, 1u);
+      // (a small input has a CTA per partition: nobody has a second one)
+      sm.ticket = R == 1 && p.ntiles <= gridDim.x ? p.ntiles : atomicAdd(&p.ws->ticket, 1u);
       sm.known = p.early_exit ? ld_relaxed_u64(reinterpret_cast<const uint64_t *>(&p.ws->errkey)) : NO_ERROR;
     }
     __syncthreads();
@@ -313,22 +336,18 @@ __device__ __forceinline__ void wtranscode(const Params &p, WSmem<Codec> &sm, Fi
     const unsigned long long known = sm.known;
     uint32_t nxt_total = 0;
     if (nxt < p.ntiles) {
-      wcount_part<Codec>(p, nxt, sm.counts[cb ^ 1]);
+      wcount_part<Codec, R>(p, nxt, sm.counts[cb ^ 1]);
       __syncthreads();
       nxt_total = wpart_total(sm.counts[cb ^ 1]);
-      if (tid == 0) {
-        publish_aggregate(p, nxt, nxt_total, epoch);
-        atomicAdd(&p.ws->total, (unsigned long long)nxt_total);
-      }
+      all_units += nxt_total;
+      if (tid == 0) publish_aggregate(p, nxt, nxt_total, epoch);
     }
+    if ((unsigned long long)cur * wide_part_bytes(R) > known) break;  // uniform over the CTA
     const uint64_t S0 = lookback_cta<XT>(p, cur, cur_total, epoch, sm.lb);
-
-    if ((unsigned long long)cur * PART_BYTES <= known) {  // uniform over the CTA
-      wconvert_part<Codec>(p, cur, sm.counts[cb], S0, sm, use, err_pos);
-      if (p.early_exit && err_pos < published) {  // rare: this thread flagged a new error
-        atomicMin(&p.ws->errkey, err_pos);
-        published = err_pos;
-      }
+    wconvert_part<Codec, R>(p, cur, sm.counts[cb], S0, sm, use, err_pos);
+    if (p.early_exit && err_pos < published) {  // rare: this thread flagged a new error
+      atomicMin(&p.ws->errkey, err_pos);
+      published = err_pos;
     }
     cur = nxt;
     cur_total = nxt_total;
@@ -337,15 +356,18 @@ __device__ __forceinline__ void wtranscode(const Params &p, WSmem<Codec> &sm, Fi
   }
   if (lane == 0) bulk_wait_all<0>();
 
-  if (!fold_and_finish<XT>(p, err_pos, true, sm.red, &sm.is_last)) return;
+  if (tid == 0) __threadfence();  // a look-back that gave up has said so before the CTA is counted
+  unsigned long long tot;
+  bool errors;
+  if (!finish_packed<XT>(p, err_pos, all_units, sm.red, &sm.is_last, &tot, &errors)) return;
   if (tid == 0) {
     WsHeader *ws = p.ws;
     const uint32_t status = *(volatile uint32_t *)&ws->status;
-    const unsigned long long key = *(volatile unsigned long long *)&ws->errkey;
-    const unsigned long long tot = *(volatile unsigned long long *)&ws->total;
+    unsigned long long key = NO_ERROR;
+    if (errors) key = *(volatile unsigned long long *)&ws->errkey;
     finalize(status, key, tot);
   }
-  reset_workspace(p);
+  reset_workspace(p, epoch);
 }
 
 // ---- explicit shared-memory stores (32-bit shared addresses) ------------------------------

@@ -432,7 +432,7 @@ __device__ __forceinline__ void transcode(const Params &p, XSmem<Codec> &sm, Fin
     const unsigned long long tot = *(volatile unsigned long long *)&ws->total;
     finalize(status, key, tot);
   }
-  reset_workspace(p);
+  reset_workspace(p, epoch);
 }
 
 // ---- several strings in one launch -----------------------------------------------------------
@@ -565,7 +565,7 @@ __device__ __forceinline__ void transcode_segments(const SegParams &q, XSmem<Cod
     r.ws = q.ws;
     r.states = q.states;
     r.max_states = q.max_states;
-    reset_workspace(r);
+    reset_workspace(r, epoch);
   }
 }
 
