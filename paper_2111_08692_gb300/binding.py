@@ -386,6 +386,11 @@ class Codec:
         if device is None:
             device = torch.cuda.current_device()
         self.device = device
+        # looked up once: a call on a small input costs less than the lookups
+        self._lib = lib()
+        self._device = torch.device("cuda", device)
+        # the current stream's handle without a Stream object (2.7 us of a 5.5 us call)
+        self._raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
         self.ctx = gbu_create(device, max_units)
         if not self.ctx:
             raise GbuError("gbu_create failed")
@@ -404,11 +409,13 @@ class Codec:
     # helpers
     def _stream(self, stream):
         if stream is None:
-            stream = self.torch.cuda.current_stream(self.device)
+            if self._raw_stream is not None:
+                return self._raw_stream(self.device)
+            return self.torch.cuda.current_stream(self._device).cuda_stream
         return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
     def new_result(self):
-        return self.torch.empty(2, dtype=self.torch.int64, device=f"cuda:{self.device}")
+        return self.torch.empty(2, dtype=self.torch.int64, device=self._device)
 
     @staticmethod
     def _ptr(t):
@@ -446,68 +453,65 @@ class Codec:
         _check(gbu_reset(self.ctx), "gbu_reset")
 
     # operations (tensors are 1-D, contiguous, on this device)
-    def validate_utf8(self, src, result=None, stream=None):
+    def _read(self, name, src, out, stream):
+        rc = getattr(self._lib, name)(self.ctx, self._ptr(src), src.numel(), out.data_ptr(), self._stream(stream))
+        if rc:
+            _check(rc, name)
+        return out
+
+    def _convert(self, name, src, dst, result, stream, cap):
         result = self.new_result() if result is None else result
-        _check(gbu_validate_utf8(self.ctx, self._ptr(src), src.numel(), result.data_ptr(),
-                                 self._stream(stream)), "gbu_validate_utf8")
+        rc = getattr(self._lib, name)(self.ctx, self._ptr(src), src.numel(), self._ptr(dst),
+                                      dst.numel() if cap is None else cap, result.data_ptr(), self._stream(stream))
+        if rc:
+            _check(rc, name)
         return result
+
+    def _new_length(self):
+        return self.torch.empty(1, dtype=self.torch.int64, device=self._device)
+
+    def validate_utf8(self, src, result=None, stream=None):
+        return self._read("gbu_validate_utf8", src, self.new_result() if result is None else result, stream)
 
     def validate_utf16le(self, src, result=None, stream=None):
-        result = self.new_result() if result is None else result
-        _check(gbu_validate_utf16le(self.ctx, self._ptr(src), src.numel(), result.data_ptr(),
-                                    self._stream(stream)), "gbu_validate_utf16le")
-        return result
+        return self._read("gbu_validate_utf16le", src, self.new_result() if result is None else result, stream)
 
     def utf16_length_from_utf8(self, src, out=None, stream=None):
-        out = self.torch.empty(1, dtype=self.torch.int64, device=f"cuda:{self.device}") if out is None else out
-        _check(gbu_utf16_length_from_utf8(self.ctx, self._ptr(src), src.numel(), out.data_ptr(),
-                                          self._stream(stream)), "gbu_utf16_length_from_utf8")
-        return out
+        return self._read("gbu_utf16_length_from_utf8", src, self._new_length() if out is None else out, stream)
 
     def utf8_length_from_utf16le(self, src, out=None, stream=None):
-        out = self.torch.empty(1, dtype=self.torch.int64, device=f"cuda:{self.device}") if out is None else out
-        _check(gbu_utf8_length_from_utf16le(self.ctx, self._ptr(src), src.numel(), out.data_ptr(),
-                                            self._stream(stream)), "gbu_utf8_length_from_utf16le")
-        return out
+        return self._read("gbu_utf8_length_from_utf16le", src, self._new_length() if out is None else out, stream)
 
     def convert_utf8_to_utf16le(self, src, dst, result=None, stream=None, cap=None):
-        result = self.new_result() if result is None else result
-        cap = dst.numel() if cap is None else cap
-        _check(gbu_convert_utf8_to_utf16le(self.ctx, self._ptr(src), src.numel(), self._ptr(dst), cap,
-                                           result.data_ptr(), self._stream(stream)),
-               "gbu_convert_utf8_to_utf16le")
-        return result
+        return self._convert("gbu_convert_utf8_to_utf16le", src, dst, result, stream, cap)
+
+    def convert_utf16le_to_utf8(self, src, dst, result=None, stream=None, cap=None):
+        return self._convert("gbu_convert_utf16le_to_utf8", src, dst, result, stream, cap)
 
     # host-synchronising forms: (status name, count) by value, the stream waited for
-    def _sync(self, fn, name, *args):
-        r = fn(self.ctx, *args)
+    def _sync(self, name, *args):
+        r = getattr(self._lib, name)(self.ctx, *args)
         return STATUS.get(r.status, r.status), int(r.count)
 
     def validate_utf8_sync(self, src, stream=None):
-        return self._sync(lib().gbu_validate_utf8_sync, "gbu_validate_utf8_sync", self._ptr(src), src.numel(),
-                          self._stream(stream))
+        return self._sync("gbu_validate_utf8_sync", self._ptr(src), src.numel(), self._stream(stream))
 
     def validate_utf16le_sync(self, src, stream=None):
-        return self._sync(lib().gbu_validate_utf16le_sync, "gbu_validate_utf16le_sync", self._ptr(src), src.numel(),
-                          self._stream(stream))
+        return self._sync("gbu_validate_utf16le_sync", self._ptr(src), src.numel(), self._stream(stream))
 
     def utf16_length_from_utf8_sync(self, src, stream=None):
-        return self._sync(lib().gbu_utf16_length_from_utf8_sync, "gbu_utf16_length_from_utf8_sync", self._ptr(src),
-                          src.numel(), self._stream(stream))
+        return self._sync("gbu_utf16_length_from_utf8_sync", self._ptr(src), src.numel(), self._stream(stream))
 
     def utf8_length_from_utf16le_sync(self, src, stream=None):
-        return self._sync(lib().gbu_utf8_length_from_utf16le_sync, "gbu_utf8_length_from_utf16le_sync",
-                          self._ptr(src), src.numel(), self._stream(stream))
+        return self._sync("gbu_utf8_length_from_utf16le_sync", self._ptr(src), src.numel(), self._stream(stream))
 
     def convert_utf8_to_utf16le_sync(self, src, dst, stream=None, cap=None):
-        cap = dst.numel() if cap is None else cap
-        return self._sync(lib().gbu_convert_utf8_to_utf16le_sync, "gbu_convert_utf8_to_utf16le_sync", self._ptr(src),
-                          src.numel(), self._ptr(dst), cap, self._stream(stream))
+        return self._sync("gbu_convert_utf8_to_utf16le_sync", self._ptr(src), src.numel(), self._ptr(dst),
+                          dst.numel() if cap is None else cap, self._stream(stream))
 
     def convert_utf16le_to_utf8_sync(self, src, dst, stream=None, cap=None):
-        cap = dst.numel() if cap is None else cap
-        return self._sync(lib().gbu_convert_utf16le_to_utf8_sync, "gbu_convert_utf16le_to_utf8_sync", self._ptr(src),
-                          src.numel(), self._ptr(dst), cap, self._stream(stream))
+        return self._sync("gbu_convert_utf16le_to_utf8_sync", self._ptr(src), src.numel(), self._ptr(dst),
+                          dst.numel() if cap is None else cap, self._stream(stream))
 
     # UTF-16BE forms: int16 tensors holding the words as they lie in memory (big-endian bytes)
     def validate_utf16be(self, src, result=None, stream=None):
@@ -675,14 +679,6 @@ class Codec:
         if not g:
             raise GbuError("gbu_graph_end failed")
         return Graph(g, self)
-
-    def convert_utf16le_to_utf8(self, src, dst, result=None, stream=None, cap=None):
-        result = self.new_result() if result is None else result
-        cap = dst.numel() if cap is None else cap
-        _check(gbu_convert_utf16le_to_utf8(self.ctx, self._ptr(src), src.numel(), self._ptr(dst), cap,
-                                           result.data_ptr(), self._stream(stream)),
-               "gbu_convert_utf16le_to_utf8")
-        return result
 
 
 def shard_cuts_host(data, P: int):

@@ -89,13 +89,21 @@ struct DeviceGuard {
 
 }  // namespace
 
+// The result of a *_sync call.  The kernel writes it straight into mapped host memory, so that the
+// call is a launch and a wait, without a copy: 8 -> 16 of 100 bytes 29 us with a copy back, 23 so.
+struct SyncSlot {
+  gbu_result res;
+  uint64_t len;
+};
+
 struct gbu_ctx {
   int device;
   uint64_t max_units;
   int num_sms;
   gbu::WsHeader *ws;   // device
-  gbu_result *sync_res; // device, right after the header: the result slot of the *_sync calls
-  uint64_t *sync_len;   // device, after sync_res: the length slot of the *_sync length calls
+  SyncSlot *sync_host;  // pinned host memory, mapped: where the *_sync calls' kernels write
+  gbu_result *sync_res; // its device addresses
+  uint64_t *sync_len;
   uint64_t *states;    // device
   uint32_t max_states;
   uint32_t wait_limit;
@@ -155,14 +163,26 @@ extern "C" gbu_ctx *gbu_create(int device, uint64_t max_units) {
     return nullptr;
   }
   c->max_states = (uint32_t)tiles;
-  // the header, then the *_sync calls' result and length slots (one allocation)
-  if (cudaMalloc(&c->ws, sizeof(gbu::WsHeader) + sizeof(gbu_result) + sizeof(uint64_t)) != cudaSuccess) {
+  if (cudaMalloc(&c->ws, sizeof(gbu::WsHeader)) != cudaSuccess) {
     delete c;
     return nullptr;
   }
-  c->sync_res = reinterpret_cast<gbu_result *>(c->ws + 1);
-  c->sync_len = reinterpret_cast<uint64_t *>(c->sync_res + 1);
+  SyncSlot *slot = nullptr;
+  if (cudaHostAlloc(&c->sync_host, sizeof(SyncSlot), cudaHostAllocMapped) != cudaSuccess) {
+    cudaFree(c->ws);
+    delete c;
+    return nullptr;
+  }
+  if (cudaHostGetDevicePointer((void **)&slot, c->sync_host, 0) != cudaSuccess) {
+    cudaFreeHost(c->sync_host);
+    cudaFree(c->ws);
+    delete c;
+    return nullptr;
+  }
+  c->sync_res = &slot->res;
+  c->sync_len = &slot->len;
   if (cudaMalloc(&c->states, (size_t)c->max_states * sizeof(uint64_t)) != cudaSuccess) {
+    cudaFreeHost(c->sync_host);
     cudaFree(c->ws);
     delete c;
     return nullptr;
@@ -175,6 +195,7 @@ extern "C" gbu_ctx *gbu_create(int device, uint64_t max_units) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, f, kernel_threads(k), smem) != cudaSuccess ||
         bps < 1) {
       cudaFree(c->states);
+      cudaFreeHost(c->sync_host);
       cudaFree(c->ws);
       delete c;
       return nullptr;
@@ -203,6 +224,7 @@ extern "C" gbu_ctx *gbu_create(int device, uint64_t max_units) {
   }
   if (!occ_ok) {
     cudaFree(c->states);
+    cudaFreeHost(c->sync_host);
     cudaFree(c->ws);
     delete c;
     return nullptr;
@@ -213,6 +235,7 @@ extern "C" gbu_ctx *gbu_create(int device, uint64_t max_units) {
   for (int m = 0; m < K_COUNT; ++m) c->batch_cfg[m] = gbu_batch_config{8, 64, 16384, 0};
   if (init_workspace(c) != GBU_OK) {
     cudaFree(c->states);
+    cudaFreeHost(c->sync_host);
     cudaFree(c->ws);
     delete c;
     return nullptr;
@@ -224,6 +247,7 @@ extern "C" void gbu_destroy(gbu_ctx *c) {
   if (!c) return;
   DeviceGuard g(c->device);
   cudaFree(c->states);
+  cudaFreeHost(c->sync_host);
   cudaFree(c->ws);
   delete c;
 }
@@ -396,9 +420,9 @@ extern "C" int gbu_convert_utf16le_to_utf8(gbu_ctx *c, const uint16_t *src, uint
 
 // ---- host-synchronising forms ---------------------------------------------------------------
 
-// Completes a *_sync call: rc is the launch status of the asynchronous call, which wrote its
-// result (or, for a length, the length) into the context's slot on `stream`.  Copies the slot
-// back and waits for the stream.
+// Completes a *_sync call: rc is the launch status of the asynchronous call, which writes its
+// result (or, for a length, the length) into the context's slot on `stream`.  Waits for the stream
+// and reads the slot.
 static gbu_result finish_sync(gbu_ctx *c, int rc, gbu_stream stream, bool length) {
   gbu_result r;
   r.status = rc;
@@ -406,21 +430,18 @@ static gbu_result finish_sync(gbu_ctx *c, int rc, gbu_stream stream, bool length
   r.count = 0;
   if (rc != GBU_OK) return r;
   DeviceGuard g(c->device);
-  uint64_t len = 0;
-  void *host = length ? (void *)&len : (void *)&r;
-  const void *dev = length ? (const void *)c->sync_len : (const void *)c->sync_res;
-  if (cudaMemcpyAsync(host, dev, length ? sizeof(len) : sizeof(r), cudaMemcpyDeviceToHost, (cudaStream_t)stream) !=
-          cudaSuccess ||
-      cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) {
+  if (cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) {
     cudaGetLastError();
     r.status = GBU_CUDA_ERROR;
-    r.reserved = 0;
-    r.count = 0;
     return r;
   }
+  const volatile SyncSlot *slot = c->sync_host;
   if (length) {
     r.status = GBU_OK;
-    r.count = len;
+    r.count = slot->len;
+  } else {
+    r.status = slot->res.status;
+    r.count = slot->res.count;
   }
   return r;
 }
