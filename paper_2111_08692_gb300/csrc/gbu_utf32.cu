@@ -19,6 +19,7 @@
 #include "gbu_chunk.cuh"
 #include "gbu_device.cuh"
 #include "gbu_kernels.h"
+#include "gbu_wide_utf8.cuh"
 #include "gbu_xcode.cuh"
 
 namespace gbu {
@@ -168,38 +169,67 @@ struct Utf32ToUtf8 {
     return n;
   }
 
-  // Encodes the chunk's units (Section 3's UTF-8 layout) into the staging buffer from index
-  // base + x0; an invalid unit flags the chunk (its bytes lie past the first error).
+  // A unit's UTF-8 bytes, the first in the lowest byte, and their number: the payload bits are spread
+  // to six per byte, the size's marker bits added, and the bytes reversed to the top (Section 3's
+  // layout).  MAX: the longest form that occurs.
+  template <int MAX>
+  __device__ __forceinline__ static uint32_t encode(uint32_t u, uint32_t &len) {
+    const bool g1 = u >= 0x80u, g2 = MAX > 2 && u >= 0x800u, g3 = MAX > 3 && u >= 0x10000u;
+    len = 1u + (g1 ? 1u : 0u) + (g2 ? 1u : 0u) + (g3 ? 1u : 0u);
+    if (MAX == 2) return g1 ? 0x80C0u | (u >> 6) | ((u & 0x3Fu) << 8) : u;
+    uint32_t x = u & 0x3Fu;
+    x |= (u << 2) & 0x3F00u;
+    x |= (u << 4) & 0x3F0000u;
+    if (MAX > 3) x |= (u << 6) & 0x07000000u;
+    x |= g3 ? 0xF0808080u : (g2 ? 0xE08080u : 0xC080u);
+    return __byte_perm(g1 ? x : u, 0u, g3 ? 0x0123u : (g2 ? 0x4012u : (g1 ? 0x4401u : 0x4440u)));
+  }
+
+  // Encodes the chunk's units into the staging buffer from index base + x0; an invalid unit flags
+  // the chunk (its bytes lie past the first error).  No branch per unit, as text mixes sizes inside
+  // a warp (64 MiB of mixed text as UTF-8: 156 us with branches, 124 so): a unit stores MAX bytes,
+  // and those it does not have are overwritten by the units after it, so only as many as those do
+  // not reach are predicated (all of them in a chunk at a buffer end).
+  template <int MAX, bool EDGE>
+  __device__ __forceinline__ static bool encode_chunk(const uint32_t (&U)[4], uint32_t o, long long c, long long lo,
+                                                      long long hi) {
+    bool bad = false;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      uint32_t len;
+      const uint32_t z = encode<MAX>(U[j], len);
+      if (EDGE && !(c + 4 * j >= lo && c + 4 * j < hi)) {
+        len = 0;
+      } else if (MAX > 2) {
+        bad = bad || utf32_bad(U[j]);
+      }
+      const uint32_t m = (1u << len) - 1u;  // bit i: byte i exists
+      const int kept = EDGE ? 0 : 4 - j;    // bytes stored in any case
+      if (kept > 0) sts_u8(o, z); else sts_u8_if_set<0>(o, z, m, 1u);
+      if (kept > 1) sts_u8(o + 1, z >> 8); else sts_u8_if_set<1>(o, z >> 8, m, 2u);
+      if (MAX > 2) {
+        if (kept > 2) sts_u8(o + 2, z >> 16); else sts_u8_if_set<2>(o, z >> 16, m, 4u);
+      }
+      if (MAX > 3) {
+        if (kept > 3) sts_u8(o + 3, z >> 24); else sts_u8_if_set<3>(o, z >> 24, m, 8u);
+      }
+      o += len;
+    }
+    return bad;
+  }
+
   __device__ __forceinline__ static Region convert(const Params &p, uint4 v, uint32_t, uint32_t, long long c,
                                                    bool edge, bool, uint8_t *st, uint32_t base, uint32_t x0,
                                                    uint32_t rtot, uint32_t, unsigned long long &err_pos) {
     const uint32_t U[4] = {v.x, v.y, v.z, v.w};
-    uint32_t o = base + x0;
-    bool bad = false;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const bool valid = !edge || (c + 4 * j >= (long long)p.off0 && c + 4 * j < (long long)p.vbytes);
-      if (!valid) continue;
-      const uint32_t u = U[j];
-      bad = bad || utf32_bad(u);
-      const uint32_t len = utf8_len_of_unit(u);
-      if (len == 1) {
-        st[o] = (uint8_t)u;
-      } else if (len == 2) {
-        st[o] = (uint8_t)(0xC0u | (u >> 6));
-        st[o + 1] = (uint8_t)(0x80u | (u & 0x3Fu));
-      } else if (len == 3) {
-        st[o] = (uint8_t)(0xE0u | (u >> 12));
-        st[o + 1] = (uint8_t)(0x80u | ((u >> 6) & 0x3Fu));
-        st[o + 2] = (uint8_t)(0x80u | (u & 0x3Fu));
-      } else {
-        st[o] = (uint8_t)(0xF0u | ((u >> 18) & 0x07u));
-        st[o + 1] = (uint8_t)(0x80u | ((u >> 12) & 0x3Fu));
-        st[o + 2] = (uint8_t)(0x80u | ((u >> 6) & 0x3Fu));
-        st[o + 3] = (uint8_t)(0x80u | (u & 0x3Fu));
-      }
-      o += len;
-    }
+    const uint32_t o = smem_addr(st) + base + x0;
+    const long long lo = p.off0, hi = (long long)p.vbytes;
+    const uint32_t top = max(max(U[0], U[1]), max(U[2], U[3]));
+    bool bad;
+    if (__any_sync(0xffffffffu, edge)) bad = encode_chunk<4, true>(U, o, c, lo, hi);
+    else if (__any_sync(0xffffffffu, top >= 0x10000u)) bad = encode_chunk<4, false>(U, o, c, lo, hi);
+    else if (__any_sync(0xffffffffu, top >= 0x800u)) bad = encode_chunk<3, false>(U, o, c, lo, hi);
+    else bad = encode_chunk<2, false>(U, o, c, lo, hi);
     if (bad && (unsigned long long)c < err_pos) err_pos = (unsigned long long)c;
     return Region{rtot, 0u, 0u, rtot};
   }
@@ -254,47 +284,39 @@ struct Utf8ToUtf32 {
     return acc >> 7;
   }
 
-  // Validates the chunk (rules 1-3 by the lead/continuation flags, rules 4-6 by the word-level
-  // byte tests) and stores one unit per leading byte, decoded from the four bytes that start
-  // there (Section 3's payload bits, most significant first).
+  // Validates the chunk and stores one unit per leading byte: the byte-plane body of the UTF-8 ->
+  // UTF-16 transcoder (gbu_wide_utf8.cuh) on four words, with the code point's third byte in a plane
+  // of its own; which leading-byte classes occur is voted per region.  (One position at a time behind
+  // a branch, this took 2054 warp instructions per KiB: 64 MiB of mixed text 171 us, of CJK 143; now
+  // 112 and 91.)
   __device__ __forceinline__ static Region convert(const Params &p, uint4 v, uint32_t prev, uint32_t next,
                                                    long long c, bool edge, bool, uint32_t *st, uint32_t base,
                                                    uint32_t x0, uint32_t rtot, uint32_t,
                                                    unsigned long long &err_pos) {
     const uint32_t W[6] = {prev, v.x, v.y, v.z, v.w, next};
-    Flags8 f[5];
+    uint32_t c3 = 0, c4 = 0;  // leading bytes E0-EF, F0-FF, also in the word before
 #pragma unroll
-    for (int k = 0; k < 5; ++k) f[k] = classify8(W[k]);
-    uint32_t err = utf8_structure_errors(f);
-    uint32_t c2 = 0, c3 = 0, c4 = 0;
-#pragma unroll
-    for (int k = 1; k <= 4; ++k) {
-      c2 |= f[k].geC0 & ~f[k].geE0;
-      c3 |= f[k].geE0 & ~f[k].geF0;
-      c4 |= f[k].geF0;
+    for (int k = 0; k < 5; ++k) {
+      const uint32_t gE = W[k] & (W[k] << 1) & (W[k] << 2) & 0x80808080u, gF = gE & (W[k] << 3);
+      c3 |= gE & ~gF;
+      c4 |= gF;
     }
-    err |= utf8_special_errors(W, f, __any_sync(0xffffffffu, c2 != 0), __any_sync(0xffffffffu, c3 != 0),
-                               __any_sync(0xffffffffu, c4 != 0));
-    uint32_t addr = base + x0;
+    const uint32_t sa = smem_addr(st) + 4 * (base + x0);
+    uint32_t bad;
+    if (__any_sync(0xffffffffu, edge)) {
+      uint32_t m = 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const uint32_t vm = edge ? byte_range_mask(c + 4 * k, p.off0, (long long)p.vbytes) : 0x80808080u;
-      const uint32_t keep = ~f[k + 1].isC & vm;  // bit 7 of each byte: a unit starts here
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if ((keep >> (8 * q + 7)) & 1u) {
-          // the four bytes from this position on
-          const uint32_t x = __byte_perm(W[k + 1], W[k + 2], 0x3210 + 0x1111 * q);
-          const uint32_t b0 = x & 0xFFu, b1 = (x >> 8) & 0x3Fu, b2 = (x >> 16) & 0x3Fu, b3 = (x >> 24) & 0x3Fu;
-          const uint32_t cp = b0 < 0x80u   ? b0
-                              : b0 < 0xE0u ? ((b0 & 0x1Fu) << 6) | b1
-                              : b0 < 0xF0u ? ((b0 & 0x0Fu) << 12) | (b1 << 6) | b2
-                                           : ((b0 & 0x07u) << 18) | (b1 << 12) | (b2 << 6) | b3;
-          st[addr++] = cp;
-        }
-      }
+      for (int i = 0; i < 16; ++i)
+        if (c + i >= (long long)p.off0 && c + i < (long long)p.vbytes) m |= 1u << i;
+      bad = Utf8ToUtf16Wide::wconvert_fast<true, true, true, 4, true, true>(W, sa, m);
+    } else if (__any_sync(0xffffffffu, c4 != 0)) {
+      bad = Utf8ToUtf16Wide::wconvert_fast<true, true, true, 4, false, true>(W, sa);
+    } else if (__any_sync(0xffffffffu, c3 != 0)) {
+      bad = Utf8ToUtf16Wide::wconvert_fast<true, true, false, 4, false, true>(W, sa);
+    } else {
+      bad = Utf8ToUtf16Wide::wconvert_fast<true, false, false, 4, false, true>(W, sa);
     }
-    if (err && (unsigned long long)c < err_pos) err_pos = (unsigned long long)c;
+    if (bad && (unsigned long long)c < err_pos) err_pos = (unsigned long long)c;
     return Region{rtot, 0u, 0u, rtot};
   }
 };

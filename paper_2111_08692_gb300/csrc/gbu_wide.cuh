@@ -393,6 +393,13 @@ __device__ __forceinline__ void sts_u16_if(uint32_t a, uint32_t v, uint32_t flag
       "h"((unsigned short)v), "r"(flags), "r"(bit)
       : "memory");
 }
+__device__ __forceinline__ void sts_u32_if(uint32_t a, uint32_t v, uint32_t flags, uint32_t bit) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t.reg .b32 t;\n\tand.b32 t, %2, %3;\n\tsetp.ne.b32 q, t, 0;\n\t"
+      "@q st.shared.u32 [%0], %1;\n\t}" ::"r"(a),
+      "r"(v), "r"(flags), "r"(bit)
+      : "memory");
+}
 // A byte at a + OFF where (flags & bit) != 0 (the address is not advanced).
 template <int OFF>
 __device__ __forceinline__ void sts_u8_if_set(uint32_t a, uint32_t v, uint32_t flags, uint32_t bit) {

@@ -129,6 +129,54 @@ struct Utf16ToUtf8Wide {
         : "memory");
   }
 
+  // The general pair route, two words per register: the forms of the other routes, chosen per
+  // 16-bit lane.  Each surrogate writes the two bytes of its own two slots, as in the route for
+  // ASCII and pairs.  Nonzero: an unpaired surrogate.  (One word at a time, with four predicated
+  // stores each, this route took 1391 warp instructions per KiB of mixed text, twice the others; 64
+  // MiB of it as UTF-16BE 131 us, now 105.  A function of its own, so that its registers do not
+  // weigh on the other routes: inlined, 1 GiB of Cyrillic took 585 us instead of 581.)
+  __device__ __noinline__ static uint32_t general_pairs(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, uint32_t w4,
+                                                        uint32_t w5, uint32_t w6, uint32_t w7, uint32_t prev,
+                                                        uint32_t next, uint32_t o) {
+    const uint32_t W[8] = {w0, w1, w2, w3, w4, w5, w6, w7};
+    uint32_t Hp = lanes16_sur(prev) & ~(prev << 5);  // first-surrogate flags of the register before
+    uint32_t before = prev, err = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const uint32_t X = W[k], A6 = X >> 6, b10 = X << 5;
+      const uint32_t S = lanes16_sur(X), Hc = S & ~b10, Lc = S & b10;
+      // pair rule: a word is a second surrogate exactly when the one before it is a first one
+      err |= Lc ^ __funnelshift_l(Hp, Hc, 16);
+      Hp = Hc;
+      const uint32_t two = lanes16_ge80(X), three = lanes16_ge800(X) & ~S;
+      const uint32_t G1 = prmt(two, 0u, 0xBB99u), G2 = prmt(three, 0u, 0xBB99u);
+      const uint32_t Hm = prmt(Hc, 0u, 0xBB99u), Lm = prmt(Lc, 0u, 0xBB99u);
+      const uint32_t T = (X & 0x03FF03FFu) + 0x00400040u;
+      const uint32_t Xp = __funnelshift_l(before, X, 16);  // each lane's word before
+      before = X;
+      const uint32_t B2 = (X & 0x003F003Fu) | 0x00800080u;
+      const uint32_t h0 = ((T >> 8) & 0x00070007u) | 0x00F000F0u, h1 = ((T >> 2) & 0x003F003Fu) | 0x00800080u;
+      const uint32_t l0 = (Xp & 0x00030003u) * 16u + ((A6 & 0x000F000Fu) | 0x00800080u);
+      uint32_t B0 = (((A6 & 0x001F001Fu) | 0x00C000C0u) & G1) | (X & ~G1);
+      B0 = ((((X >> 12) & 0x000F000Fu) | 0x00E000E0u) & G2) | (B0 & ~G2);
+      B0 = (h0 & Hm) | (B0 & ~Hm);
+      B0 = (l0 & Lm) | (B0 & ~Lm);
+      uint32_t B1 = (((A6 & 0x003F003Fu) | 0x00800080u) & G2) | (B2 & ~G2);
+      B1 = (h1 & Hm) | (B1 & ~Hm);
+      sts_123m<0x8000u>(o, two, three, B0, B1, B2);
+      sts_123m<0x80000000u>(o, two, three, B0 >> 16, B1 >> 16, B2 >> 16);
+    }
+    // the lane's last word against the one after it
+    const uint32_t Ln = lanes16_sur(next) & (next << 5);
+    err |= (Hp >> 31) ^ ((Ln >> 15) & 1u);
+    // a pair cut by the region's end: lane 31 also writes its second half
+    if ((threadIdx.x & 31) == 31 && (Hp >> 31) && is_low16(next & 0xFFFFu)) {
+      sts_u8(o, 0x80u | ((w7 >> 16 & 3u) << 4) | ((next >> 6) & 0xFu));
+      sts_u8(o + 1, 0x80u | (next & 0x3Fu));
+    }
+    return err;
+  }
+
   __device__ __forceinline__ static Region wconvert(const Params &p, const uint32_t W[8], uint32_t prev,
                                                     uint32_t next, long long c, bool edge, bool inside, uint8_t *st,
                                                     uint32_t base, uint32_t x0, uint32_t rtot, uint32_t rflags,
@@ -271,33 +319,7 @@ struct Utf16ToUtf8Wide {
       if (err && (unsigned long long)c < err_pos) err_pos = (unsigned long long)c;
       return g;
     }
-    bool err = false;
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const uint32_t w = word(W, j);
-      const uint32_t wp = j > 0 ? word(W, j - 1) : u0, wn = j < 15 ? word(W, j + 1) : u17;
-      const bool g1 = w >= 0x80u, g2 = w >= 0x800u;
-      const bool hs = is_high16(w), ls = is_low16(w);
-      const bool pair = hs && is_low16(wn);
-      const bool follows = ls && is_high16(wp);
-      err |= (hs && !pair) || (ls && !follows);
-      // the word's bytes: a pair's four, nothing for a pair's second word, else its one to
-      // three (a lone surrogate takes the three-byte form)
-      const uint32_t c6 = w & 0x3Fu, t6 = w >> 6;
-      const uint32_t t = (w & 0x3FFu) + 0x40u;  // a pair's code point >> 10
-      const uint32_t b0 = pair ? 0xF0u | (t >> 8) : (g2 ? 0xE0u + (w >> 12) : (g1 ? 0xC0u + t6 : w));
-      const uint32_t b1 = pair ? 0x80u | ((t >> 2) & 0x3Fu) : (g2 ? 0x80u | (t6 & 0x3Fu) : 0x80u + c6);
-      const uint32_t b2 = pair ? 0x80u | ((t & 3u) << 4) | ((wn >> 6) & 0xFu) : 0x80u + c6;
-      const uint32_t nb = pair ? 4u : (follows ? 0u : 1u + (g1 ? 1u : 0u) + (g2 ? 1u : 0u));
-      // nb = 0..4 bytes: byte i is stored where nb > i, i.e. where bit i of m = 0xF >> (4 - nb)
-      // is set (tested by the fused stores)
-      const uint32_t m = 0xFu >> (4u - nb);
-      sts_u8_if_set<0>(o, b0, m, 1u);
-      sts_u8_if_set<1>(o, b1, m, 2u);
-      sts_u8_if_set<2>(o, b2, m, 4u);
-      sts_u8_if_set<3>(o, 0x80u | (wn & 0x3Fu), m, 8u);
-      o += (hs || ls) ? 2u : 1u + (g1 ? 1u : 0u) + (g2 ? 1u : 0u);
-    }
+    const uint32_t err = general_pairs(W[0], W[1], W[2], W[3], W[4], W[5], W[6], W[7], prev, next, o);
     if (err && (unsigned long long)c < err_pos) err_pos = (unsigned long long)c;
     return g;
   }

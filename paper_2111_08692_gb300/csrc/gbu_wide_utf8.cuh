@@ -145,8 +145,9 @@ struct Utf8ToUtf16Wide {
   // place of one word (a four-byte leading byte of two), the count the count pass gave the lane.
   // NW: the words of the lane (W[1..NW]).  EXACT: the lane may hold bytes outside its string (m: one
   // bit per byte inside) and other strings' words lie next to the lane's, so every word is stored
-  // under its predicate and a lane never writes past the words it counts.
-  template <bool H2, bool H3, bool H4, int NW = 8, bool EXACT = false>
+  // under its predicate and a lane never writes past the words it counts.  U32: one 32-bit unit (the
+  // code point) per leading byte instead, its third byte in a plane of its own.
+  template <bool H2, bool H3, bool H4, int NW = 8, bool EXACT = false, bool U32 = false>
   __device__ __forceinline__ static uint32_t wconvert_fast(const uint32_t (&W)[NW + 2], uint32_t sa, uint32_t m = 0) {
     // with a single class present, every byte >= C0 is a leading byte of that class; without
     // H4 there is no byte >= F0
@@ -193,7 +194,7 @@ struct Utf8ToUtf16Wide {
       }
 
       // byte planes of the output words
-      uint32_t L = w, H = 0, Lls = 0, Hls = 0;
+      uint32_t L = w, H = 0, Lls = 0, Hls = 0, U = 0;
       uint32_t S2 = 0;
       if (H3 || H4) S2 = __funnelshift_r(w, wn, 16);
       if (H2) {
@@ -210,7 +211,13 @@ struct Utf8ToUtf16Wide {
         L = (L3 & M3) | (L & ~M3);
         H = (H3v & M3) | (H & ~M3);
       }
-      if (H4) {
+      if (H4 && U32) {
+        // 11110abc 10defghi 10jk.... 10......: U = abc de, H = fghi jk.., L = the last eight bits
+        const uint32_t S3 = __funnelshift_r(w, wn, 24), M4 = byte_mask(gF);
+        L = (((S2 & 0x03030303u) * 64u + (S3 & 0x3F3F3F3Fu)) & M4) | (L & ~M4);
+        H = (((S1 & 0x0F0F0F0Fu) * 16u + ((S2 >> 2) & 0x0F0F0F0Fu)) & M4) | (H & ~M4);
+        U = ((w & 0x07070707u) * 4u + ((S1 >> 4) & 0x03030303u)) & M4;
+      } else if (H4) {
         const uint32_t S3 = __funnelshift_r(w, wn, 24);
         const uint32_t M4 = byte_mask(gF);
         // second surrogate: DC00 | (third byte & 0F) << 6 | (fourth byte & 3F)
@@ -228,6 +235,22 @@ struct Utf8ToUtf16Wide {
       }
       // stage the words (2 bytes per leading byte, 4 where it takes two words)
       const uint32_t lead = EXACT ? n & nibble_flags(m, k - 1) : n;
+      if (U32) {
+        const uint32_t step = lead >> 5;
+        // two positions' low halves, then each with its third byte (below 20: its sign gives the zero)
+        const uint32_t P[2] = {__byte_perm(L, H, 0x5140), __byte_perm(L, H, 0x7362)};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const uint32_t bit = 0x80u << (8 * j), ones = 0x01010101u >> (32 - 8 * j - (j == 0 ? 8 : 0));
+          const uint32_t at = j == 0 ? sa : __dp4a(step, ones, sa);
+          const uint32_t lo = (j & 1) ? 0x32u : 0x10u, u = 4u + (uint32_t)j;
+          const uint32_t unit = prmt(P[j >> 1], U, lo | u << 8 | (8u + u) << 12);
+          if (!EXACT && (k < NW || j < 1)) sts_u32(at, unit);
+          else sts_u32_if(at, unit, lead, bit);
+        }
+        if (k < NW) sa = __dp4a(step, 0x01010101u, sa);
+        continue;
+      }
       const uint32_t step = H4 ? (lead >> 6) + (gF >> 6) : lead >> 6;
       constexpr int FREE = H4 ? 1 : 2;  // the last word's positions that a leading byte always follows
 #pragma unroll
