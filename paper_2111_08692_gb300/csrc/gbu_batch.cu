@@ -329,15 +329,23 @@ __device__ __forceinline__ uint32_t words_to_utf8(const uint32_t (&W)[6], uint32
 }
 
 // A lane's chunk of UTF-8 (W[1..4]): its UTF-16 words, and the leading-byte classes present.
-__device__ __forceinline__ uint32_t chunk_units8(const uint32_t (&W)[6], uint32_t m, bool classes, uint32_t &flags) {
+// convert: the words as the conversion stores them (the second surrogate of a four-byte sequence at
+// the byte after its leading byte), else the length formula.
+__device__ __forceinline__ uint32_t chunk_units8(const uint32_t (&W)[6], uint32_t m, bool convert, uint32_t &flags) {
   uint32_t n = 0, c2 = 0, c3 = 0, c4 = 0;
+  uint32_t pF = W[0] & (W[0] * 2u) & (W[0] * 4u) & (W[0] * 8u) & 0x80808080u;
 #pragma unroll
   for (int k = 1; k <= 4; ++k) {
     const uint32_t w = W[k], s1 = w * 2u;
     const uint32_t g = w & s1 & 0x80808080u, gE = g & (w * 4u), gF = gE & (w * 8u);
-    n = __dp4a((~w | s1) & nibble_flags(m, k - 1), 0x01010101u, n);
-    n = __dp4a(gF, 0x01010101u, n);
-    if (classes) {
+    if (convert) {
+      n = __dp4a((~w | s1 | __funnelshift_l(pF, gF, 8)) & nibble_flags(m, k - 1), 0x01010101u, n);
+      pF = gF;
+    } else {
+      n = __dp4a((~w | s1) & nibble_flags(m, k - 1), 0x01010101u, n);
+      n = __dp4a(gF, 0x01010101u, n);
+    }
+    if (convert) {
       c2 |= g & ~gE;
       c3 |= gE & ~gF;
       c4 |= gF;

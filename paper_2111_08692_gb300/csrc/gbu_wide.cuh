@@ -21,6 +21,8 @@
 //   struct Codec {
 //     using Out = uint8_t or uint16_t;
 //     static constexpr uint32_t WSTAGE;           // staged units per warp buffer
+//     static constexpr bool CARRY;                // gives_word(lane's last word): the lane's last byte
+//                                                 // gives the next lane one of the units counted here
 //     static constexpr uint32_t ASCII_MASK;       // nonzero in an input word: a unit >= 0x80
 //     static constexpr uint32_t LANE_UNITS;       // units out of 32 bytes of ASCII input
 //     static constexpr uint32_t WREGION_UNITS;    // units out of an all-ASCII region
@@ -126,6 +128,9 @@ __device__ __forceinline__ void wcount_partition(const Params &p, uint32_t part,
   uint32_t v[R][8];
 #pragma unroll
   for (int r = 0; r < R; ++r) load32(p, s0 + (long long)r * WREGION + WLANE * lane, inside, keep, v[r]);
+  uint32_t gives = 0;  // CARRY: the byte before the region gives its first lane a word
+  // (only INSIDE leaves a word to spare before the slice)
+  if (Codec::CARRY) gives = Codec::gives_word(INSIDE ? ldg_word(p.base + s0 - 4) : load_word_checked(p, s0 - 4));
   bool slice_ascii = false;
   if (INSIDE) {
     uint32_t any = 0;
@@ -152,8 +157,18 @@ __device__ __forceinline__ void wcount_partition(const Params &p, uint32_t part,
         const long long c = s0 + (long long)(r + q) * WREGION + WLANE * lane;
         const bool edge = !inside && (c < lo || c + (long long)WLANE > hi);
         a[q] = Codec::wcount(p, v[r + q], c, edge, f[q]);
+        if (Codec::CARRY) {
+          const bool last = Codec::gives_word(v[r + q][7]);
+          if (__any_sync(0xffffffffu, last) || gives) {  // uniform over the warp
+            uint32_t in = __shfl_up_sync(0xffffffffu, (uint32_t)last, 1);
+            if (lane == 0) in = gives;
+            gives = __shfl_sync(0xffffffffu, (uint32_t)last, 31);
+            a[q] += in - (uint32_t)last;
+          }
+          a[q] = min(a[q], WLANE);  // more only where a rule is broken
+        }
       }
-      // two regions per scan: a region has at most 32 x 64 units
+      // two regions per scan: a region has at most 32 x 48 units
       const uint32_t x = a[0] | (a[1] << 16);
       uint32_t incl;
       const uint32_t x_first = __shfl_sync(0xffffffffu, x, 0);

@@ -27,6 +27,9 @@ struct Utf16ToUtf8Wide {
   static constexpr uint32_t WSTAGE = 3 * 512 + 32;
   static_assert(3 * 512 + 2 + 15 + 1 <= WSTAGE, "staging buffer too small");
 
+  static constexpr bool CARRY = false;
+  __device__ __forceinline__ static bool gives_word(uint32_t) { return false; }
+
   static constexpr uint32_t F_SUR = Narrow::F_SUR;
   static constexpr uint32_t F_THREE = Narrow::F_THREE;
   static constexpr uint32_t F_WIDE = Narrow::F_WIDE;

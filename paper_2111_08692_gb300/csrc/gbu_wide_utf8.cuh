@@ -11,14 +11,16 @@
 //     the one or two bytes after it (S1, S2 = the byte stream moved by one and two positions):
 //       two bytes   110abcde 10fghijk      -> H = 00000abc,  L = de fghijk
 //       three bytes 1110abcd 10efghij 10k.. -> H = abcd efgh, L = ij k.....
-//     and for a four-byte sequence the two surrogates (the first as D7C0 + the code point's
-//     bits 20-10, the second as DC00 + its bits 9-0);
+//     and for a four-byte sequence the two surrogates: the leading byte gives the first (D7C0 +
+//     the code point's bits 20-10), the byte after it the second (DC00 + bits 9-0), which seen
+//     from there is the three-byte form's expression with other upper bits, so that a position
+//     never gives more than one word (with both at the leading byte and the second one stored
+//     under its own predicate: 512 MiB of emoji text 569 us, now 525; of mixed text 769, now 721);
 //   * PRMT interleaves H and L into 16-bit words, which go to consecutive places of the staging
 //     buffer, through 32-bit shared-memory addresses.  Every position stores its word, whether it
 //     is a leading byte's or not, at the place the next leading byte's word takes: what a
 //     continuation byte writes is overwritten by the lane's next leading byte.  Only the lane's
-//     last positions, which no leading byte may follow, store under a predicate (as do second
-//     surrogates).  The places of a word's four positions are byte dot products of its leading
+//     last positions, which no leading byte may follow, store under a predicate.  The places of a word's four positions are byte dot products of its leading
 //     flags with one to four ones, added to the running address: the multiply pipe makes them,
 //     and of the test, store and add that every position cost before, on the integer pipe that
 //     bounds the kernel, only the store is left (CJK: 756 to 723 warp instructions per KiB; 1 GiB
@@ -52,12 +54,12 @@ __device__ __forceinline__ uint32_t plane_word(uint32_t L, uint32_t H, int j) {
 struct Utf8ToUtf16Wide {
   using Out = uint16_t;
   using Narrow = Utf8ToUtf16;
-  // A valid 1 KiB region yields at most 1024 words, +1 for a four-byte leading byte in its last
-  // byte.  A lane that breaks a rule can count up to 64 words while every lane before it is
-  // valid, so a lane's own staging always fits: 32 x 31 + 1 + 64, plus 7 words of alignment
-  // offset, <= WSTAGE.  Words past the buffer can only come after the first error.
+  // A region yields at most 1024 words (one per position), plus 7 words of alignment offset and the
+  // place after the last word, which continuation bytes may write to after an error.
   static constexpr uint32_t WSTAGE = 1024 + 48;
-  static_assert(32 * 31 + 1 + 64 + 7 <= WSTAGE, "staging buffer too small");
+  static_assert(1024 + 7 + 1 <= WSTAGE, "staging buffer too small");
+  static constexpr bool CARRY = true;  // a lane's last byte can give a word to the next lane
+  __device__ __forceinline__ static bool gives_word(uint32_t w) { return w >= 0xF0000000u; }
 
   static constexpr uint32_t F_NONASCII = Narrow::F_NONASCII;
   static constexpr uint32_t F_C2 = Narrow::F_C2;
@@ -141,8 +143,8 @@ struct Utf8ToUtf16Wide {
   // region that lies inside the buffer and whose output fits the staging buffer, and stages
   // their words from shared address sa on; returns nonzero when a rule is broken.  H2 / H3 /
   // H4: leading bytes C0-DF / E0-EF / F0-FF occur in the region or in bytes 1-3 of the word
-  // before it (the code for an absent class is left out).  Each non-continuation byte takes the
-  // place of one word (a four-byte leading byte of two), the count the count pass gave the lane.
+  // before it (the code for an absent class is left out).  Each non-continuation byte and each byte
+  // after a leading byte F0-FF takes the place of one word, the count the count pass gave the lane.
   // NW: the words of the lane (W[1..NW]).  EXACT: the lane may hold bytes outside its string (m: one
   // bit per byte inside) and other strings' words lie next to the lane's, so every word is stored
   // under its predicate and a lane never writes past the words it counts.  U32: one 32-bit unit (the
@@ -172,6 +174,7 @@ struct Utf8ToUtf16Wide {
       if (H4) gF = ONE ? g : gE & (w << 3);        // >= F0
       // rules 1-3: a byte is a continuation exactly when a leading byte 1, 2 or 3 back wants it
       uint32_t req = __funnelshift_l(pg, g, 8);
+      const uint32_t F1 = H4 ? __funnelshift_l(pF, gF, 8) : 0u;  // the byte after a leading byte F0-FF
       if (H3 || H4) req |= __funnelshift_l(pE, gE, 16);
       if (H4) req |= __funnelshift_l(pF, gF, 24);
       bad |= (req ^ n) ^ 0x80808080u;
@@ -194,7 +197,7 @@ struct Utf8ToUtf16Wide {
       }
 
       // byte planes of the output words
-      uint32_t L = w, H = 0, Lls = 0, Hls = 0, U = 0;
+      uint32_t L = w, H = 0, U = 0;
       uint32_t S2 = 0;
       if (H3 || H4) S2 = __funnelshift_r(w, wn, 16);
       if (H2) {
@@ -204,12 +207,15 @@ struct Utf8ToUtf16Wide {
         L = (L2 & M2) | (L & ~M2);
         H = H2v & M2;
       }
+      uint32_t L3 = 0, H3v = 0;
+      if (H3 || (H4 && !U32)) {
+        L3 = (S1 & 0x03030303u) * 64u + (S2 & 0x3F3F3F3Fu);
+        H3v = (S1 >> 2) & 0x0F0F0F0Fu;
+      }
       if (H3) {
-        const uint32_t L3 = (S1 & 0x03030303u) * 64u + (S2 & 0x3F3F3F3Fu);
-        const uint32_t H3v = wF * 16u + ((S1 >> 2) & 0x0F0F0F0Fu);
         const uint32_t M3 = byte_mask(ONE ? g : (H4 ? gE & ~gF : gE));
         L = (L3 & M3) | (L & ~M3);
-        H = (H3v & M3) | (H & ~M3);
+        H = ((wF * 16u + H3v) & M3) | (H & ~M3);
       }
       if (H4 && U32) {
         // 11110abc 10defghi 10jk.... 10......: U = abc de, H = fghi jk.., L = the last eight bits
@@ -218,23 +224,21 @@ struct Utf8ToUtf16Wide {
         H = (((S1 & 0x0F0F0F0Fu) * 16u + ((S2 >> 2) & 0x0F0F0F0Fu)) & M4) | (H & ~M4);
         U = ((w & 0x07070707u) * 4u + ((S1 >> 4) & 0x03030303u)) & M4;
       } else if (H4) {
-        const uint32_t S3 = __funnelshift_r(w, wn, 24);
-        const uint32_t M4 = byte_mask(gF);
+        const uint32_t M4 = byte_mask(gF), M1 = byte_mask(F1);
         // second surrogate: DC00 | (third byte & 0F) << 6 | (fourth byte & 3F)
-        Lls = (S2 & 0x03030303u) * 64u + (S3 & 0x3F3F3F3Fu);
-        Hls = ((S2 >> 2) & 0x03030303u) | 0xDCDCDCDCu;
+        L = (L3 & M1) | (L & ~M1);
+        H = (((H3v & 0x03030303u) | 0xDCDCDCDCu) & M1) | (H & ~M1);
         // first surrogate: D7C0 + ((lead & 7) << 8 | Y), Y = (second & 3F) << 2 | (third >> 4) & 3;
         // Y is cleared outside F0-FF positions, so the per-byte sums below carry at most into
-        // the byte after a leading byte (a continuation position, which stores nothing)
+        // the byte after a leading byte, where M4 drops them
         const uint32_t Y = ((S1 & 0x3F3F3F3Fu) * 4u + ((S2 >> 4) & 0x03030303u)) & M4;
         const uint32_t cy = ((Y | (Y << 1)) >> 7) & 0x01010101u;  // Y >= 0x40: the low byte wraps
-        const uint32_t Lhs = Y + 0xC0C0C0C0u;
-        const uint32_t Hhs = (w & 0x07070707u) + cy + 0xD7D7D7D7u;
-        L = (Lhs & M4) | (L & ~M4);
-        H = (Hhs & M4) | (H & ~M4);
+        L = ((Y + 0xC0C0C0C0u) & M4) | (L & ~M4);
+        H = (((w & 0x07070707u) + cy + 0xD7D7D7D7u) & M4) | (H & ~M4);
       }
-      // stage the words (2 bytes per leading byte, 4 where it takes two words)
-      const uint32_t lead = EXACT ? n & nibble_flags(m, k - 1) : n;
+      // stage the words
+      const uint32_t all = U32 ? n : n | F1;  // the positions that give one
+      const uint32_t lead = EXACT ? all & nibble_flags(m, k - 1) : all;
       if (U32) {
         const uint32_t step = lead >> 5;
         // two positions' low halves, then each with its third byte (below 20: its sign gives the zero)
@@ -251,15 +255,14 @@ struct Utf8ToUtf16Wide {
         if (k < NW) sa = __dp4a(step, 0x01010101u, sa);
         continue;
       }
-      const uint32_t step = H4 ? (lead >> 6) + (gF >> 6) : lead >> 6;
-      constexpr int FREE = H4 ? 1 : 2;  // the last word's positions that a leading byte always follows
+      const uint32_t step = lead >> 6;
+      constexpr int FREE = 2;  // the last word's positions that another word of the lane always follows
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const uint32_t bit = 0x80u << (8 * j), ones = 0x01010101u >> (32 - 8 * j - (j == 0 ? 8 : 0));
         const uint32_t at = j == 0 ? sa : __dp4a(step, ones, sa);
         if (!EXACT && (k < NW || j < FREE)) sts_u16(at, plane_word(L, H, j));
         else sts_u16_if(at, plane_word(L, H, j), lead, bit);
-        if (H4) sts_u16_if(at + 2, plane_word(Lls, Hls, j), gF, bit);
       }
       if (k < NW) sa = __dp4a(step, 0x01010101u, sa);
     }
@@ -299,16 +302,16 @@ struct Utf8ToUtf16Wide {
       }
       return Region{1024u, 0u, 0u, 1024u};
     }
-    if (inside && base + rtot < WSTAGE) {
-      const uint32_t Wx[10] = {prev, W[0], W[1], W[2], W[3], W[4], W[5], W[6], W[7], next};
+    const uint32_t Wx[10] = {prev, W[0], W[1], W[2], W[3], W[4], W[5], W[6], W[7], next};
+    const uint32_t sa = sbase + 2 * (base + x0);
+    uint32_t bad;
+    if (inside) {
       // the leading-byte classes: the region's own (from the count pass) and those of bytes
       // 1-3 of the word before it (a sequence starting there reaches into the region, and the
       // structure test reads those bytes)
       const uint32_t pc = lane == 0 ? Narrow::lead_classes(prev, 0x80808000u) : 0u;
       const uint32_t cls = rflags | __shfl_sync(0xffffffffu, pc, 0);
       const bool h2 = cls & F_C2, h3 = cls & F_C3, h4 = cls & F_C4;
-      const uint32_t sa = sbase + 2 * (base + x0);
-      uint32_t bad;
       if (h4) {
         bad = (h2 || h3) ? wconvert_fast<true, true, true>(Wx, sa) : wconvert_fast<false, false, true>(Wx, sa);
       } else if (h3) {
@@ -316,28 +319,17 @@ struct Utf8ToUtf16Wide {
       } else {
         bad = h2 ? wconvert_fast<true, false, false>(Wx, sa) : wconvert_fast<true, true, true>(Wx, sa);
       }
-      if (bad && (unsigned long long)c < err_pos) err_pos = (unsigned long long)c;
-      return Region{rtot, 0u, 0u, rtot};
+    } else {
+      // a region at a buffer end: all classes, the bytes outside masked off (with the 16-byte
+      // general path inlined here, 512 MiB of ASCII took 292 us instead of 273, 100 MB of CJK 114
+      // instead of 100: its code and registers weighed on the paths that run)
+      const long long a = (long long)p.off0 - c, b = (long long)p.vbytes - c;
+      const uint32_t from = a <= 0 ? 0u : (a >= 32 ? 32u : (uint32_t)a), to = b <= 0 ? 0u : (b >= 32 ? 32u : (uint32_t)b);
+      const uint32_t below = to == 32 ? 0xFFFFFFFFu : (1u << to) - 1u;
+      bad = wconvert_fast<true, true, true, 8, true>(Wx, sa, from == 32 ? 0u : below & (0xFFFFFFFFu << from));
     }
-    const Narrow::General r = wconvert_general(p, make_uint4(W[0], W[1], W[2], W[3]),
-                                               make_uint4(W[4], W[5], W[6], W[7]), prev, next, c, edge, st, base,
-                                               x0, rtot, err_pos);
-    err_pos = r.err_pos;
-    return r.g;
-  }
-
-  // A region at a buffer end (or one whose output overflows the staging buffer, which only
-  // happens after an error): the 16-byte general path of the narrow codec on each half of the
-  // lane's bytes (A, B).
-  __device__ __forceinline__ static Narrow::General wconvert_general(const Params &p, uint4 A, uint4 B, uint32_t prev,
-                                                                  uint32_t next, long long c, bool edge, uint16_t *st,
-                                                                  uint32_t base, uint32_t x0, uint32_t rtot,
-                                                                  unsigned long long err_pos) {
-    const long long lo = p.off0, hi = (long long)p.vbytes;
-    uint32_t fa;
-    const uint32_t na = Narrow::count(p, A, c, edge, fa);
-    const Narrow::General ra = Narrow::convert_general_body(lo, hi, A, prev, B.x, c, edge, st, base, x0, rtot, err_pos, WSTAGE);
-    return Narrow::convert_general_body(lo, hi, B, A.w, next, c + 16, edge, st, base, x0 + na, rtot, ra.err_pos, WSTAGE);
+    if (bad && (unsigned long long)c < err_pos) err_pos = (unsigned long long)c;
+    return Region{rtot, 0u, 0u, rtot};
   }
 };
 
