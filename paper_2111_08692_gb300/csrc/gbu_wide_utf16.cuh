@@ -63,38 +63,37 @@ struct Utf16ToUtf8Wide {
   // summed by byte dot products.
   __device__ __forceinline__ static uint32_t wcount(const Params &p, const uint32_t W[8], long long c, bool edge,
                                                     uint32_t &flags) {
-    if (!edge) {
-      uint32_t any = 0;
+    uint32_t any = 0;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) any |= W[k];
-      flags = 0;
-      if ((any & ASCII_MASK) == 0) return 16;  // all ASCII
-      uint32_t a80 = 0, a800 = 0, sub = 0;
+    for (int k = 0; k < 8; ++k) any |= W[k];
+    flags = 0;
+    if (!edge && (any & ASCII_MASK) == 0) return 16;  // all ASCII
+    uint32_t a80 = 0, a800 = 0, sub = 0;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const uint32_t hb = __byte_perm(W[2 * i], W[2 * i + 1], 0x7531);
-        const uint32_t lb = __byte_perm(W[2 * i], W[2 * i + 1], 0x6420);
-        const uint32_t g80 = (((hb & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | hb | lb) & 0x80808080u;
-        const uint32_t g800 = (((hb & 0x78787878u) + 0x78787878u) | hb) & 0x80808080u;
-        const uint32_t t = (hb & 0xF8F8F8F8u) ^ 0xD8D8D8D8u;
-        const uint32_t sr = ~(((t & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | t) & 0x80808080u;
-        a80 = __dp4a(g80, 0x01010101u, a80);
-        a800 = __dp4a(g800, 0x01010101u, a800);
-        sub = __dp4a(sr, 0x01010101u, sub);
-      }
-      // every surrogate is >= 0x800: a80 - sub counts the words >= 0x80 that are not surrogates
-      flags = (sub ? F_SUR : 0u) | (a800 ? F_THREE : 0u) | (a80 != sub ? F_WIDE : 0u);
-      return 16u + ((a80 + a800 - sub) >> 7);
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t hb = __byte_perm(W[2 * i], W[2 * i + 1], 0x7531);
+      const uint32_t lb = __byte_perm(W[2 * i], W[2 * i + 1], 0x6420);
+      const uint32_t g80 = (((hb & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | hb | lb) & 0x80808080u;
+      const uint32_t g800 = (((hb & 0x78787878u) + 0x78787878u) | hb) & 0x80808080u;
+      const uint32_t t = (hb & 0xF8F8F8F8u) ^ 0xD8D8D8D8u;
+      const uint32_t sr = ~(((t & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | t) & 0x80808080u;
+      a80 = __dp4a(g80, 0x01010101u, a80);
+      a800 = __dp4a(g800, 0x01010101u, a800);
+      sub = __dp4a(sr, 0x01010101u, sub);
     }
-    flags = F_SUR | F_THREE | F_WIDE;
-    uint32_t cnt = 0;
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const uint32_t w = (W[j >> 1] >> (16 * (j & 1))) & 0xFFFFu;
-      const bool valid = c + 2 * j >= (long long)p.off0 && c + 2 * j < (long long)p.vbytes;
-      cnt += valid ? len8_of_word(w) : 0u;
-    }
-    return cnt;
+    // every surrogate is >= 0x800: a80 - sub counts the words >= 0x80 that are not surrogates
+    flags = (sub ? F_SUR : 0u) | (a800 ? F_THREE : 0u) | (a80 != sub ? F_WIDE : 0u);
+    // words outside the input read as zero
+    const uint32_t words = edge ? (uint32_t)__popc(valid_bits(p, c)) / 2u : 16u;
+    return words + ((a80 + a800 - sub) >> 7);
+  }
+
+  // Bit i: byte i of the 32 bytes at position c lies inside the input.
+  __device__ __forceinline__ static uint32_t valid_bits(const Params &p, long long c) {
+    const long long a = (long long)p.off0 - c, b = (long long)p.vbytes - c;
+    const uint32_t from = a <= 0 ? 0u : (a >= 32 ? 32u : (uint32_t)a), to = b <= 0 ? 0u : (b >= 32 ? 32u : (uint32_t)b);
+    const uint32_t below = to == 32 ? 0xFFFFFFFFu : (1u << to) - 1u;
+    return from == 32 ? 0u : below & (0xFFFFFFFFu << from);
   }
 
   // Word j (0..15) of the lane.
@@ -138,9 +137,11 @@ struct Utf16ToUtf8Wide {
   // stores each, this route took 1391 warp instructions per KiB of mixed text, twice the others; 64
   // MiB of it as UTF-16BE 131 us, now 105.  A function of its own, so that its registers do not
   // weigh on the other routes: inlined, 1 GiB of Cyrillic took 585 us instead of 581.)
+  // EDGE: m has a bit per byte inside the input; words outside read as zero and are not stored.
+  template <bool EDGE>
   __device__ __noinline__ static uint32_t general_pairs(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, uint32_t w4,
                                                         uint32_t w5, uint32_t w6, uint32_t w7, uint32_t prev,
-                                                        uint32_t next, uint32_t o) {
+                                                        uint32_t next, uint32_t o, uint32_t m) {
     const uint32_t W[8] = {w0, w1, w2, w3, w4, w5, w6, w7};
     uint32_t Hp = lanes16_sur(prev) & ~(prev << 5);  // first-surrogate flags of the register before
     uint32_t before = prev, err = 0;
@@ -166,8 +167,20 @@ struct Utf16ToUtf8Wide {
       B0 = (l0 & Lm) | (B0 & ~Lm);
       uint32_t B1 = (((A6 & 0x003F003Fu) | 0x00800080u) & G2) | (B2 & ~G2);
       B1 = (h1 & Hm) | (B1 & ~Hm);
-      sts_123m<0x8000u>(o, two, three, B0, B1, B2);
-      sts_123m<0x80000000u>(o, two, three, B0 >> 16, B1 >> 16, B2 >> 16);
+      if (EDGE) {
+        const uint32_t v = ((m >> (4 * k)) & 1u) << 15 | ((m >> (4 * k + 2)) & 1u) << 31;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const uint32_t bit = j ? 0x80000000u : 0x8000u;
+          sts_u8_if_set<0>(o, B0 >> (16 * j), v, bit);
+          sts_u8_if_set<1>(o, B1 >> (16 * j), two, bit);
+          sts_u8_if_set<2>(o, B2 >> (16 * j), three, bit);
+          o += (v & bit ? 1u : 0u) + (two & bit ? 1u : 0u) + (three & bit ? 1u : 0u);
+        }
+      } else {
+        sts_123m<0x8000u>(o, two, three, B0, B1, B2);
+        sts_123m<0x80000000u>(o, two, three, B0 >> 16, B1 >> 16, B2 >> 16);
+      }
     }
     // the lane's last word against the one after it
     const uint32_t Ln = lanes16_sur(next) & (next << 5);
@@ -186,18 +199,7 @@ struct Utf16ToUtf8Wide {
                                                     unsigned long long &err_pos) {
     const int lane = threadIdx.x & 31;
     const uint32_t sbase = smem_addr(st);
-    if (!inside) {
-      // a region at a buffer end: the 16-byte generic path of the narrow codec on each half
-      // (a pair cut by the region's start is judged by lane 0's first half, one cut by its end
-      // by lane 31's second half)
-      const uint4 A = make_uint4(W[0], W[1], W[2], W[3]), B = make_uint4(W[4], W[5], W[6], W[7]);
-      uint32_t fa;
-      const uint32_t na = Narrow::count(p, A, c, edge, fa);
-      const Region ga = Narrow::convert_generic(p, A, prev, W[4], c, edge, st, base, x0, rtot, err_pos);
-      const Region gb = Narrow::convert_generic(p, B, W[3], next, c + 16, edge, st, base, x0 + na, rtot, err_pos);
-      return Region{rtot, ga.skip, gb.extra, rtot};
-    }
-    if (rtot == 512u) {
+    if (inside && rtot == 512u) {
       // 512 words and 512 bytes: every word is ASCII (Section 4's ASCII route)
       const uint4 b = narrow16(W);
       const uint32_t x = base + 16 * lane;
@@ -218,7 +220,7 @@ struct Utf16ToUtf8Wide {
     }
     Region g{rtot, 0u, 0u, rtot};
     uint32_t o = sbase + base + x0;
-    if (!(rflags & (F_SUR | F_THREE))) {
+    if (inside && !(rflags & (F_SUR | F_THREE))) {
       // Only words below 0x800 (Section 4's one-and-two-byte route), two words per register:
       // per 16-bit lane, the first byte is the word itself or C0 | w >> 6, the second 80 | w & 3F.
 #pragma unroll
@@ -233,7 +235,7 @@ struct Utf16ToUtf8Wide {
       }
       return g;
     }
-    if (!(rflags & F_SUR)) {
+    if (inside && !(rflags & F_SUR)) {
       // No surrogate in the region: every word is a character of one to three bytes, two words
       // per register.  Per 16-bit lane: the first byte is w, C0 | w >> 6 or E0 | w >> 12; the
       // second 80 | w & 3F (two bytes) or 80 | (w >> 6) & 3F (three); the third 80 | w & 3F.
@@ -253,16 +255,15 @@ struct Utf16ToUtf8Wide {
       }
       return g;
     }
-    // Surrogates present.  A first surrogate followed by a second one writes all four bytes
-    // of the pair (its two slots and its partner's); the second writes nothing.  A pair cut
-    // by the region's end is written by this region (2 bytes past its end), a pair cut by
-    // its start by the previous region.
+    // Surrogates present (or a buffer end).  Each surrogate writes the two bytes of its own two
+    // slots; the second half of a pair cut by the region's end is written by this region too (2
+    // bytes past its end), and not stored by the region after it.
     const uint32_t u0 = prev >> 16, u17 = next & 0xFFFFu;
     const bool cut_start = is_low16(word(W, 0)) && is_high16(u0);
     const bool cut_end = is_high16(word(W, 15)) && is_low16(u17);
     g.skip = __shfl_sync(0xffffffffu, cut_start ? 2u : 0u, 0);
     g.extra = __shfl_sync(0xffffffffu, cut_end ? 2u : 0u, 31);
-    if (!(rflags & F_WIDE)) {
+    if (inside && !(rflags & F_WIDE)) {
       // Only ASCII words and surrogates (emoji-heavy text), two words per register at a time.
       // An ASCII word writes its byte.  Each surrogate writes the two bytes of its own two
       // slots: a first surrogate (code point bits 20-12) F0 | t >> 8 and 80 | (t >> 2) & 3F with
@@ -322,7 +323,10 @@ struct Utf16ToUtf8Wide {
       if (err && (unsigned long long)c < err_pos) err_pos = (unsigned long long)c;
       return g;
     }
-    const uint32_t err = general_pairs(W[0], W[1], W[2], W[3], W[4], W[5], W[6], W[7], prev, next, o);
+    // any text, and the regions at a buffer end
+    const uint32_t err =
+        inside ? general_pairs<false>(W[0], W[1], W[2], W[3], W[4], W[5], W[6], W[7], prev, next, o, 0u)
+               : general_pairs<true>(W[0], W[1], W[2], W[3], W[4], W[5], W[6], W[7], prev, next, o, valid_bits(p, c));
     if (err && (unsigned long long)c < err_pos) err_pos = (unsigned long long)c;
     return g;
   }
