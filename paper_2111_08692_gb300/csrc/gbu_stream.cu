@@ -243,11 +243,14 @@ __global__ void __launch_bounds__(STREAM_THREADS, stream_min_blocks<KMODE>()) st
 
 // UTF-8 validation: a warp streams 4 KiB warp tiles, four regions of 1 KiB, a lane 32 consecutive
 // bytes of each (one 256-bit load; the source base is rounded to 32 bytes), judged on bit planes
-// (gbu_planes.cuh).  A region without a byte >= 80 takes one vote.  Bound by HBM for ASCII, by the
-// integer pipe else (CJK: 76% busy, 180 warp instructions per KiB; the byte-wise routes before took
-// 280).  Each region's registers are loaded with the warp's next tile as soon as the region is
-// judged, so that three regions' judgement covers the load.  1 GiB of CJK: 440 us before (2.4
-// TB/s), 266 with all loads of a tile issued together, 261 so.
+// (gbu_planes.cuh).  A region without a byte >= 80 takes one vote; one without a byte >= E0 is judged
+// four bytes at a time (1 GiB of Latin or Cyrillic: 267 us on the planes, 252 by the byte-wise
+// kernel before them, 221 so), tried only while the warp's last region was such a one (the route
+// costs CJK and emoji 4% even so: 272 to 284 and 290 to 302).  Bound by HBM for ASCII, by the integer
+// pipe else (the planes on CJK: 76% busy, 180 warp instructions per KiB; the byte-wise route before
+// took 280).  Each region's registers are loaded with the warp's next tile as soon as the region is
+// judged, so that three regions' judgement covers the load.  1 GiB of CJK: 440 us by the byte-wise
+// kernel (2.4 TB/s); on the planes alone 266 with all loads of a tile issued together, 261 so.
 constexpr int V8_REGIONS = (int)(WT_BYTES / 1024u);
 
 // The lane's 32 bytes at virtual position c (bytes outside the input read as zero).
@@ -274,6 +277,7 @@ __global__ void __launch_bounds__(STREAM_THREADS, 3) validate8_kernel(const Para
   const bool early = p.early_exit != 0;
   uint32_t known = 0xFFFFFFFFu, it = 0;
   long long wt = (long long)blockIdx.x * ST_WARPS + warp;
+  bool high = false;  // the warp's last judged region had a byte >= E0: go to the planes at once
   uint32_t W[V8_REGIONS][8], pre = 0, post = 0;
   if (wt < (long long)p.ntiles) {
     const long long t0 = wt * WT_BYTES;
@@ -300,16 +304,19 @@ __global__ void __launch_bounds__(STREAM_THREADS, 3) validate8_kernel(const Para
 #pragma unroll
       for (int k = 0; k < 8; ++k) any |= W[r][k];
       if (__any_sync(0xffffffffu, (any & 0x80808080u) != 0 || (lane == 31 && pending != 0))) {
-        const uint32_t after = r + 1 < V8_REGIONS ? W[r + 1 < V8_REGIONS ? r + 1 : r][0] : post;
-        const uint32_t next = __shfl_sync(0xffffffffu, lane == 0 ? after : W[r][0], (lane + 1) & 31);
-        const uint32_t err = utf8_plane_errors(
-            W[r],
-            [&](uint32_t out) {
-              const uint32_t wanted = __shfl_sync(0xffffffffu, lane == 31 ? pending : out, (lane + 31) & 31);
-              pending = out;
-              return wanted;
-            },
-            next);
+        auto exchange = [&](uint32_t out) {
+          const uint32_t wanted = __shfl_sync(0xffffffffu, lane == 31 ? pending : out, (lane + 31) & 31);
+          pending = out;
+          return wanted;
+        };
+        uint32_t err;
+        if (high || !utf8_two_byte_errors(W[r], exchange, err)) {
+          const uint32_t after = r + 1 < V8_REGIONS ? W[r + 1 < V8_REGIONS ? r + 1 : r][0] : post;
+          const uint32_t next = __shfl_sync(0xffffffffu, lane == 0 ? after : W[r][0], (lane + 1) & 31);
+          bool any3;
+          err = utf8_plane_errors(W[r], exchange, next, any3);
+          high = __any_sync(0xffffffffu, any3);
+        }
         em |= err ? 1u << r : 0u;
       } else {
         pending = 0;

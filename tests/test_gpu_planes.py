@@ -57,3 +57,24 @@ def test_lengths_around_tiles(n, shift):
         assert int(codec.utf8_length_from_utf16be(be[shift:]).item()) == oracle.utf8_length_from_utf16le(u16)
     finally:
         codec.close()
+
+
+@pytest.mark.parametrize("shift", [0, 5])
+@pytest.mark.parametrize("at", [32, 1022, 1024, 2048, 4094, 4096, 8192])
+def test_sequences_in_two_byte_text(at, shift):
+    """Regions of two-byte characters are judged without the planes: every sequence inside them."""
+    import torch
+    from paper_2111_08692_gb300 import Codec, result_tuple
+    codec = Codec(0, max_units=1 << 20)
+    try:
+        for lead in range(at, at + 4):
+            for seq in SEQUENCES + ["\u0416".encode(), "\u6c34".encode(), "\U0001f600".encode()]:
+                pairs = (lead - shift) // 2
+                head = "\u044f".encode() * pairs + b"a" * (lead - shift - 2 * pairs)
+                data = np.frombuffer(head + seq + "\u00e9".encode() * 6000, np.uint8)
+                buf = torch.zeros(data.size + shift, dtype=torch.uint8, device="cuda")
+                buf[shift:] = torch.from_numpy(data.copy())
+                got = result_tuple(codec.validate_utf8(buf[shift:]))
+                assert got == oracle.validate_utf8(data), (lead, seq.hex())
+    finally:
+        codec.close()
