@@ -90,8 +90,9 @@ void gbu_set_wait_limit(gbu_ctx *ctx, uint32_t rounds);
 void gbu_debug_skip_publish(gbu_ctx *ctx, int64_t tile);
 /* Early exit on invalid input (on by default).  The single-buffer validation calls and
  * transcoders publish the position of a flagged chunk as soon as a thread finds one; work
- * that lies wholly past it is skipped (validation stops reading, a transcoder still counts
- * and chains such a partition but does not convert it).  Results are identical either way,
+ * that lies wholly past it is skipped (validation stops reading; a transcoder between UTF-8 and
+ * UTF-16 stops too, one of UTF-32 still counts and chains such a partition but does not convert
+ * it).  Results are identical either way,
  * since the first error and the output of the valid prefix never lie past a flagged chunk;
  * only the time to reach them changes.  enable = 0 scans every input to the end (used to
  * time full scans).  Not in the paper, whose kernels process blocks in order and can stop at
@@ -130,9 +131,8 @@ int gbu_convert_utf16le_to_utf8(gbu_ctx *ctx, const uint16_t *src, uint64_t n, u
  *   validate / convert: the gbu_result the asynchronous call would have written;
  *   lengths: {GBU_OK, length}.
  * A launch failure returns {that status (GBU_BAD_ARGUMENT, GBU_CUDA_ERROR), 0}; a NULL ctx
- * returns {GBU_BAD_ARGUMENT, 0}.  The result travels through a slot of the context's workspace
- * (device memory) and one device-to-host copy, so calls on one context must not overlap, as
- * for the asynchronous calls. */
+ * returns {GBU_BAD_ARGUMENT, 0}.  The kernel writes the result into a slot of the context in mapped
+ * host memory, so calls on one context must not overlap, as for the asynchronous calls. */
 gbu_result gbu_validate_utf8_sync(gbu_ctx *ctx, const uint8_t *src, uint64_t n, gbu_stream stream);
 gbu_result gbu_validate_utf16le_sync(gbu_ctx *ctx, const uint16_t *src, uint64_t n, gbu_stream stream);
 gbu_result gbu_utf16_length_from_utf8_sync(gbu_ctx *ctx, const uint8_t *src, uint64_t n, gbu_stream stream);
