@@ -247,7 +247,9 @@ int gbu_per_string_loop(gbu_ctx *ctx, int op, const void *src, const uint64_t *o
  * strings_per_claim consecutive strings at a time (more in a large batch, fewer in one that
  * would leave SMs idle); a warp packs its share of them, 32 chunks of 16 bytes per step, except
  * that strings of at least long_bytes input bytes are handled afterwards by the whole CTA
- * (warps_per_cta x 512 bytes per step). */
+ * (warps_per_cta x 512 bytes per step).  A batch of no more strings than the device runs CTAs at
+ * once has a CTA for each string, and then, unless the geometry was set or tuned, strings of 1536
+ * bytes on are handled by their whole CTA. */
 typedef struct {
   int32_t warps_per_cta;      /* 4, 8 or 16 (default 8) */
   uint32_t strings_per_claim; /* 1 .. 1024 (default 64) */

@@ -7,6 +7,7 @@
 #include <atomic>
 #include <vector>
 
+#include "gbu_batch_plan.h"
 #include "gbu_device.cuh"
 #include "gbu_internal.h"
 #include "gbu_kernels.h"
@@ -114,6 +115,7 @@ struct gbu_ctx {
   int scan_blocks_per_sm;
   int seg_blocks_per_sm[2];             // several-string transcoders: 8 -> 16, 16 -> 8
   gbu_batch_config batch_cfg[K_COUNT];  // launch geometry of the batched kernels
+  bool batch_chosen[K_COUNT];           // set by the caller or the tuner
   std::atomic<uint64_t> launches;
   uint64_t capture_start;               // launches when the current graph capture began
 };
@@ -207,7 +209,7 @@ extern "C" gbu_ctx *gbu_create(int device, uint64_t max_units) {
   for (int m = 0; m < K_COUNT && occ_ok; ++m)
     for (int w = 0; w < 3 && occ_ok; ++w) {
       int bps = 0;
-      occ_ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, gbu::batch_kernel_ptr(m, kWarps[w]),
+      occ_ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, gbu::batch_kernel_ptr(m, kWarps[w], false),
                                                              kWarps[w] * 32, 0) == cudaSuccess && bps >= 1;
       c->batch_blocks_per_sm[m][w] = bps;
     }
@@ -229,8 +231,8 @@ extern "C" gbu_ctx *gbu_create(int device, uint64_t max_units) {
     delete c;
     return nullptr;
   }
-  // Strings from 16 KiB on go to a whole CTA: packed, one of them keeps a warp busy for 32 steps,
-  // and the CTA's narrow regions cost more per byte (a million log-normal strings, 8 -> 16 / 16 -> 8:
+  // In a large batch (gbu_batch_plan.h) strings from 16 KiB on go to a whole CTA: packed, one of them
+  // keeps a warp busy for 32 steps, and the CTA's narrow regions cost more per byte (a million log-normal strings, 8 -> 16 / 16 -> 8:
   // 461 / 530 us with the line at 4 KiB, 412 / 476 at 8 KiB, 387 / 438 at 16 KiB, 401 / 457 at 32).
   for (int m = 0; m < K_COUNT; ++m) c->batch_cfg[m] = gbu_batch_config{8, 64, 16384, 0};
   if (init_workspace(c) != GBU_OK) {
@@ -684,10 +686,10 @@ static int batch_check_config(const gbu_batch_config &b) {
   return GBU_OK;
 }
 
-// Launches batched mode m over B strings with geometry cfg.
-static int batch_launch(gbu_ctx *c, int m, const gbu_batch_config &cfg, const void *src, const uint64_t *off,
-                        uint64_t B, void *dst, const uint64_t *dst_off, gbu_result *results, uint64_t *lens,
-                        gbu_stream stream, const gbu::StringDesc *desc = nullptr) {
+// Launches batched mode m over B strings with geometry cfg (chosen: not the library's defaults).
+static int batch_launch(gbu_ctx *c, int m, const gbu_batch_config &cfg, bool chosen, const void *src,
+                        const uint64_t *off, uint64_t B, void *dst, const uint64_t *dst_off, gbu_result *results,
+                        uint64_t *lens, gbu_stream stream, const gbu::StringDesc *desc = nullptr) {
   if (B == 0) return GBU_OK;  // nothing to write
   gbu::BatchParams bp;
   memset(&bp, 0, sizeof(bp));
@@ -700,19 +702,14 @@ static int batch_launch(gbu_ctx *c, int m, const gbu_batch_config &cfg, const vo
   bp.results = results;
   bp.lens = lens;
   bp.ws = c->ws;
-  // a batch with fewer claims than SMs is cut finer, down to a string per warp
-  bp.grab = cfg.strings_per_claim;
-  const uint64_t fine = B / (uint64_t)c->num_sms;
-  if (fine < bp.grab) bp.grab = fine > (uint64_t)cfg.warps_per_cta ? (uint32_t)fine : (uint32_t)cfg.warps_per_cta;
-  if (bp.grab > cfg.strings_per_claim) bp.grab = cfg.strings_per_claim;
-  bp.long_bytes = cfg.long_bytes;
+  const gbu::BatchPlan plan =
+      gbu::batch_plan(B, (uint32_t)c->num_sms, (uint32_t)c->batch_blocks_per_sm[m][warps_index(cfg.warps_per_cta)],
+                      cfg.warps_per_cta, cfg.strings_per_claim, cfg.long_bytes, chosen);
+  bp.group = plan.group;
+  bp.long_bytes = plan.long_bytes;
   DeviceGuard g(c->device);
-  uint64_t grid = (uint64_t)c->num_sms * (uint64_t)c->batch_blocks_per_sm[m][warps_index(cfg.warps_per_cta)];
-  const uint64_t claims = (B + bp.grab - 1) / bp.grab;
-  if (claims < grid) grid = claims;
-  if (grid < 1) grid = 1;
   void *args[] = {(void *)&bp};
-  cudaError_t e = cudaLaunchKernel(gbu::batch_kernel_ptr(m, cfg.warps_per_cta), dim3((unsigned)grid),
+  cudaError_t e = cudaLaunchKernel(gbu::batch_kernel_ptr(m, cfg.warps_per_cta, plan.per_cta), dim3(plan.grid),
                                    dim3(cfg.warps_per_cta * 32), args, 0, (cudaStream_t)stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -743,8 +740,8 @@ static int batch_call(gbu_ctx *c, int m, const void *src, const uint64_t *off, u
   int rc = batch_args(c, m, src, off, B, dst, dst_off, out);
   if (rc != GBU_OK) return rc;
   const bool length = m == K_L8 || m == K_L16;
-  return batch_launch(c, m, c->batch_cfg[m], src, off, B, dst, dst_off, length ? nullptr : (gbu_result *)out,
-                      length ? (uint64_t *)out : nullptr, stream);
+  return batch_launch(c, m, c->batch_cfg[m], c->batch_chosen[m], src, off, B, dst, dst_off,
+                      length ? nullptr : (gbu_result *)out, length ? (uint64_t *)out : nullptr, stream);
 }
 
 extern "C" int gbu_validate_utf8_batched(gbu_ctx *c, const uint8_t *src, const uint64_t *off, uint64_t B,
@@ -823,6 +820,7 @@ extern "C" int gbu_set_batch_config(gbu_ctx *c, int op, const gbu_batch_config *
   const int rc = batch_check_config(*cfg);
   if (rc != GBU_OK) return rc;
   c->batch_cfg[op] = *cfg;
+  c->batch_chosen[op] = true;
   return GBU_OK;
 }
 
@@ -855,11 +853,11 @@ extern "C" int gbu_tune_batched(gbu_ctx *c, int op, const void *src, const uint6
     for (int gi = 0; gi < 4 && rc == GBU_OK; ++gi)
       for (int li = 0; li < 4 && rc == GBU_OK; ++li) {
         const gbu_batch_config cand{kWarps[w], kGrab[gi], kLong[li], 0.0f};
-        rc = batch_launch(c, op, cand, src, off, B, dst, dst_off, results, lens, stream);
+        rc = batch_launch(c, op, cand, true, src, off, B, dst, dst_off, results, lens, stream);
         float t_best = -1.0f;
         for (int r = 0; r < reps && rc == GBU_OK; ++r) {
           if (cudaEventRecord(e0, (cudaStream_t)stream) != cudaSuccess) rc = GBU_CUDA_ERROR;
-          if (rc == GBU_OK) rc = batch_launch(c, op, cand, src, off, B, dst, dst_off, results, lens, stream);
+          if (rc == GBU_OK) rc = batch_launch(c, op, cand, true, src, off, B, dst, dst_off, results, lens, stream);
           if (rc == GBU_OK && cudaEventRecord(e1, (cudaStream_t)stream) != cudaSuccess) rc = GBU_CUDA_ERROR;
           float ms = 0.0f;
           if (rc == GBU_OK && (cudaEventSynchronize(e1) != cudaSuccess ||
@@ -875,7 +873,8 @@ extern "C" int gbu_tune_batched(gbu_ctx *c, int op, const void *src, const uint6
   if (rc == GBU_OK) {
     best.tuned_ms = best_ms;
     c->batch_cfg[op] = best;
-    rc = batch_launch(c, op, best, src, off, B, dst, dst_off, results, lens, stream);
+    c->batch_chosen[op] = true;
+    rc = batch_launch(c, op, best, true, src, off, B, dst, dst_off, results, lens, stream);
     if (rc == GBU_OK && cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) rc = GBU_CUDA_ERROR;
   }
   cudaEventDestroy(e0);
@@ -955,8 +954,8 @@ int gbu_internal_batch_desc(gbu_ctx *c, int op, const gbu::StringDesc *desc, uin
                             gbu_stream stream) {
   if (!c || op < 0 || op >= K_COUNT || op == K_L8 || op == K_L16) return GBU_BAD_ARGUMENT;
   if (B > 0 && (!desc || !results)) return GBU_BAD_ARGUMENT;
-  return batch_launch(c, op, c->batch_cfg[op], nullptr, nullptr, B, nullptr, nullptr, results, nullptr, stream,
-                      desc);
+  return batch_launch(c, op, c->batch_cfg[op], c->batch_chosen[op], nullptr, nullptr, B, nullptr, nullptr, results,
+                      nullptr, stream, desc);
 }
 
 int gbu_internal_partitions(int op, const void *src, uint64_t n) {

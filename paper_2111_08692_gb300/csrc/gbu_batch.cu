@@ -18,6 +18,7 @@
 //     its output starts.
 // The chunks' analysis is that of the single-buffer kernels, so each string's result is the one a
 // single-buffer call on it gives.
+// A batch of no more strings than resident CTAs gives each a CTA of its own (gbu_batch_plan.h).
 // Strings never wait on one another, so nothing spins.  Output offsets of a transcoding come
 // from the caller's dst_off (for example the exclusive scan of the batched lengths).
 // What bounds it: instruction issue on the integer pipe (63-65% busy in the conversions), then the
@@ -26,6 +27,7 @@
 // the library's autotuner from timed candidates.
 #include <stdint.h>
 
+#include "gbu_batch_plan.h"
 #include "gbu_chunk.cuh"
 #include "gbu_codec_utf16.cuh"
 #include "gbu_codec_utf8.cuh"
@@ -77,8 +79,7 @@ struct __align__(128) BatchSmem {
   static constexpr int SW = BatchTraits<MODE>::CONVERT ? NWARPS : 1;
   static constexpr uint32_t SU = BatchTraits<MODE>::CONVERT ? BatchCodec<MODE>::C::STAGE : 8u;
   Out staging[SW][2][SU];
-  // 32 strings per group; 16 where 16 warps' groups and staging buffers share 48 KB
-  static constexpr int GROUP = NWARPS == 16 ? 16 : 32;
+  static constexpr int GROUP = (int)batch_group_max(NWARPS);
   PackedStrings<GROUP> packed[NWARPS];
   uint32_t rcount[2][NWARPS];        // long strings: units of each warp's region in a step
   unsigned long long red[NWARPS];    // long strings: per-warp error position or count
@@ -654,20 +655,26 @@ __device__ __forceinline__ void cta_string(const BatchParams &bp, uint64_t i, Ba
 }
 
 // Resident warps per SM the register budget is held to: 32 (64 registers a thread), 24 for the
-// UTF-8 -> UTF-16 transcoder (80).
-template <int MODE, int NWARPS>
+// UTF-8 -> UTF-16 transcoder (80).  FEW: CTA i handles string i and nothing else, together or with its
+// first warp (an instance of its own: the same test inside the claim loop spilled more registers there,
+// and a million strings took 1,090 us instead of 1,084).
+template <int MODE, int NWARPS, bool FEW>
 __global__ void __launch_bounds__(NWARPS * 32, (MODE == B_C8 ? 24 : 32) / NWARPS) batch_kernel(const BatchParams bp) {
   using T = BatchTraits<MODE>;
   using Smem = BatchSmem<MODE, NWARPS>;
   __shared__ Smem sm;
   const int lane = threadIdx.x & 31;
   uint32_t use = 0;  // regions staged by this warp (picks its staging buffer)
-  // Strings per warp and claim: a full group where every warp gets several, else an equal share
-  // of the claim the geometry names.
+  if (FEW) {
+    const uint64_t bytes = string_units(bp, blockIdx.x) * T::IN_UNIT;
+    if (bytes >= bp.long_bytes || bytes >= PACK_LIMIT) cta_string<MODE, NWARPS>(bp, blockIdx.x, sm, use);
+    else if (threadIdx.x < 32) packed_strings<MODE, NWARPS>(bp, blockIdx.x, 1, sm);
+    if (T::CONVERT && lane == 0) bulk_wait_all<0>();
+    return;
+  }
   constexpr uint32_t FULL = Smem::GROUP;
   static_assert(BATCH_LONGS >= 2 * FULL * NWARPS, "room for every warp's group past the stop mark");
-  const uint32_t share = max(1u, min(FULL, bp.grab / NWARPS));
-  const uint32_t group = bp.B >= (uint64_t)gridDim.x * (4u * FULL * NWARPS) ? FULL : share;
+  const uint32_t group = bp.group;  // at most FULL
   if (threadIdx.x == 0) sm.nlong = sm.more = 0;
   __syncthreads();
   while (true) {
@@ -788,22 +795,22 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_u64_kernel(const ScanParams
 // ---- host-side handles -------------------------------------------------------------------
 
 template <int MODE>
-static const void *batch_ptr_for(int nwarps) {
+static const void *batch_ptr_for(int nwarps, bool few) {
   switch (nwarps) {
-    case 4: return (const void *)batch_kernel<MODE, 4>;
-    case 16: return (const void *)batch_kernel<MODE, 16>;
-    default: return (const void *)batch_kernel<MODE, 8>;
+    case 4: return few ? (const void *)batch_kernel<MODE, 4, true> : (const void *)batch_kernel<MODE, 4, false>;
+    case 16: return few ? (const void *)batch_kernel<MODE, 16, true> : (const void *)batch_kernel<MODE, 16, false>;
+    default: return few ? (const void *)batch_kernel<MODE, 8, true> : (const void *)batch_kernel<MODE, 8, false>;
   }
 }
 
-const void *batch_kernel_ptr(int mode, int nwarps) {
+const void *batch_kernel_ptr(int mode, int nwarps, bool few) {
   switch (mode) {
-    case B_V8: return batch_ptr_for<B_V8>(nwarps);
-    case B_L16: return batch_ptr_for<B_L16>(nwarps);
-    case B_C8: return batch_ptr_for<B_C8>(nwarps);
-    case B_V16: return batch_ptr_for<B_V16>(nwarps);
-    case B_L8: return batch_ptr_for<B_L8>(nwarps);
-    default: return batch_ptr_for<B_C16>(nwarps);
+    case B_V8: return batch_ptr_for<B_V8>(nwarps, few);
+    case B_L16: return batch_ptr_for<B_L16>(nwarps, few);
+    case B_C8: return batch_ptr_for<B_C8>(nwarps, few);
+    case B_V16: return batch_ptr_for<B_V16>(nwarps, few);
+    case B_L8: return batch_ptr_for<B_L8>(nwarps, few);
+    default: return batch_ptr_for<B_C16>(nwarps, few);
   }
 }
 

@@ -102,7 +102,7 @@ struct BatchParams {
   gbu_result *results;       // validation, transcoding: B results
   uint64_t *lens;            // length functions: B lengths
   WsHeader *ws;              // claim counter (ticket) and completion counter (done)
-  uint32_t grab;             // strings per claim
+  uint32_t group;            // strings a warp claims at a time
   uint32_t long_bytes;       // strings of at least this many input bytes go to a whole CTA
 };
 

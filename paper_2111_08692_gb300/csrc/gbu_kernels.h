@@ -41,8 +41,9 @@ const void *utf16_to_utf8_segments_kernel_ptr();
 size_t utf8_to_utf16_segments_smem_bytes();
 size_t utf16_to_utf8_segments_smem_bytes();
 
-// batched kernels (mode: BatchMode; nwarps: 4, 8 or 16 warps per CTA) and the u64 scan
-const void *batch_kernel_ptr(int mode, int nwarps);
+// batched kernels (mode: BatchMode; nwarps: 4, 8 or 16 warps per CTA; few: the instance with one CTA per
+// string) and the u64 scan
+const void *batch_kernel_ptr(int mode, int nwarps, bool few);
 const void *scan_kernel_ptr();
 uint32_t scan_tile_items();
 int scan_threads();
