@@ -244,10 +244,12 @@ int gbu_per_string_loop(gbu_ctx *ctx, int op, const void *src, const uint64_t *o
                         const uint64_t *dst_off, gbu_result *results, gbu_stream stream);
 
 /* Launch geometry of a batched operation.  A CTA of warps_per_cta warps claims
- * strings_per_claim consecutive strings at a time (more in a large batch, fewer in one that
- * would leave SMs idle); a warp packs its share of them, 32 chunks of 16 bytes per step, except
- * that strings of at least long_bytes input bytes are handled afterwards by the whole CTA
- * (warps_per_cta x 512 bytes per step).  A batch of no more strings than the device runs CTAs at
+ * strings_per_claim consecutive strings, of which each warp takes its share (at least one, at most
+ * 32, or 16 with 16 warps); a warp packs its share, 32 chunks of 16 bytes per step, except that
+ * strings of at least long_bytes input bytes are handled afterwards by the whole CTA (warps_per_cta
+ * x 512 bytes per step).  strings_per_claim is a wish: in a batch that would leave SMs idle the share
+ * is smaller, and in one that gives every resident warp four times the largest share (about 600,000
+ * strings) it is the largest.  A batch of no more strings than the device runs CTAs at
  * once has a CTA for each string, and then, unless the geometry was set or tuned, strings of 1536
  * bytes on are handled by their whole CTA. */
 typedef struct {
@@ -261,7 +263,8 @@ int gbu_get_batch_config(const gbu_ctx *ctx, int op, gbu_batch_config *cfg);
 int gbu_set_batch_config(gbu_ctx *ctx, int op, const gbu_batch_config *cfg); /* checks ranges */
 /* Autotuner: runs operation `op` on the given batch (arguments as for the batched call of
  * that operation; `out` is results or lens) for each candidate geometry (warps 4/8/16 x
- * claims of 8/32/128/512 strings x long-string thresholds of 2/4/8/16 KiB), one untimed and
+ * claims of 1/4/16/32 strings per warp x long-string thresholds of 2/4/8/16/32 KiB, without those
+ * that come to the same launch on this batch), one untimed and
  * `reps` timed launches each (CUDA events on `stream`), keeps the fastest in the context and
  * writes it to *chosen (may be NULL).  The last launch uses the chosen geometry, so the
  * outputs are valid.  Synchronous; not capturable. */

@@ -837,9 +837,8 @@ extern "C" int gbu_tune_batched(gbu_ctx *c, int op, const void *src, const uint6
   const bool length = op == K_L8 || op == K_L16;
   gbu_result *results = length ? nullptr : (gbu_result *)out;
   uint64_t *lens = length ? (uint64_t *)out : nullptr;
-  static const int kWarps[3] = {4, 8, 16};
-  static const uint32_t kGrab[4] = {8, 32, 128, 512};
-  static const uint32_t kLong[4] = {2048, 4096, 8192, 16384};
+  gbu::BatchCandidate cands[gbu::BATCH_CANDIDATES];
+  const int ncands = gbu::batch_candidates(B, (uint32_t)c->num_sms, c->batch_blocks_per_sm[op], cands);
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess) return GBU_CUDA_ERROR;
   if (cudaEventCreate(&e1) != cudaSuccess) {
@@ -849,27 +848,24 @@ extern "C" int gbu_tune_batched(gbu_ctx *c, int op, const void *src, const uint6
   gbu_batch_config best = c->batch_cfg[op];
   float best_ms = -1.0f;
   rc = GBU_OK;
-  for (int w = 0; w < 3 && rc == GBU_OK; ++w)
-    for (int gi = 0; gi < 4 && rc == GBU_OK; ++gi)
-      for (int li = 0; li < 4 && rc == GBU_OK; ++li) {
-        const gbu_batch_config cand{kWarps[w], kGrab[gi], kLong[li], 0.0f};
-        rc = batch_launch(c, op, cand, true, src, off, B, dst, dst_off, results, lens, stream);
-        float t_best = -1.0f;
-        for (int r = 0; r < reps && rc == GBU_OK; ++r) {
-          if (cudaEventRecord(e0, (cudaStream_t)stream) != cudaSuccess) rc = GBU_CUDA_ERROR;
-          if (rc == GBU_OK) rc = batch_launch(c, op, cand, true, src, off, B, dst, dst_off, results, lens, stream);
-          if (rc == GBU_OK && cudaEventRecord(e1, (cudaStream_t)stream) != cudaSuccess) rc = GBU_CUDA_ERROR;
-          float ms = 0.0f;
-          if (rc == GBU_OK && (cudaEventSynchronize(e1) != cudaSuccess ||
-                               cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
-            rc = GBU_CUDA_ERROR;
-          if (rc == GBU_OK && (t_best < 0.0f || ms < t_best)) t_best = ms;
-        }
-        if (rc == GBU_OK && (best_ms < 0.0f || t_best < best_ms)) {
-          best_ms = t_best;
-          best = cand;
-        }
-      }
+  for (int i = 0; i < ncands && rc == GBU_OK; ++i) {
+    const gbu_batch_config cand{cands[i].warps, cands[i].claim, cands[i].long_bytes, 0.0f};
+    rc = batch_launch(c, op, cand, true, src, off, B, dst, dst_off, results, lens, stream);
+    float t_best = -1.0f;
+    for (int r = 0; r < reps && rc == GBU_OK; ++r) {
+      if (cudaEventRecord(e0, (cudaStream_t)stream) != cudaSuccess) rc = GBU_CUDA_ERROR;
+      if (rc == GBU_OK) rc = batch_launch(c, op, cand, true, src, off, B, dst, dst_off, results, lens, stream);
+      if (rc == GBU_OK && cudaEventRecord(e1, (cudaStream_t)stream) != cudaSuccess) rc = GBU_CUDA_ERROR;
+      float ms = 0.0f;
+      if (rc == GBU_OK && (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
+        rc = GBU_CUDA_ERROR;
+      if (rc == GBU_OK && (t_best < 0.0f || ms < t_best)) t_best = ms;
+    }
+    if (rc == GBU_OK && (best_ms < 0.0f || t_best < best_ms)) {
+      best_ms = t_best;
+      best = cand;
+    }
+  }
   if (rc == GBU_OK) {
     best.tuned_ms = best_ms;
     c->batch_cfg[op] = best;

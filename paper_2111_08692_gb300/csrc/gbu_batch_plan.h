@@ -42,7 +42,9 @@ inline BatchPlan batch_plan(uint64_t B, uint32_t sms, uint32_t ctas_per_sm, int 
     return p;
   }
   // A batch with fewer claims than SMs is cut finer, down to a string per warp; a warp takes its share
-  // of a claim, and full groups where every warp gets several.
+  // of a claim, and a full group where every warp gets several, whatever the claim: each claim is an
+  // atomic on one address (a million strings, 8 -> 16 / 16 -> 8, us, by a warp's share: 1 string 1,058 /
+  // 922, 4 489 / 507, 8 427 / 446, 16 385 / 416, 32 380 / 412).
   uint64_t grab = claim;
   const uint64_t fine = B / sms > (uint64_t)warps ? B / sms : (uint64_t)warps;
   if (fine < grab) grab = fine;
@@ -54,6 +56,36 @@ inline BatchPlan batch_plan(uint64_t B, uint32_t sms, uint32_t ctas_per_sm, int 
   p.per_cta = false;
   p.long_bytes = long_bytes;
   return p;
+}
+
+struct BatchCandidate {
+  int warps;
+  uint32_t claim, long_bytes;
+};
+constexpr int BATCH_CANDIDATES = 60;
+
+// The geometries that the tuner times on a batch of B strings, without those that come to the launch of
+// an earlier one: warps 4, 8 and 16, a warp's share of a claim 1, 4, 16 and 32 strings, and long strings
+// from 2 to 32 KiB.  ctas_per_sm: resident CTAs per SM for 4, 8 and 16 warps.  Returns their number.
+inline int batch_candidates(uint64_t B, uint32_t sms, const int (&ctas_per_sm)[3], BatchCandidate (&out)[BATCH_CANDIDATES]) {
+  const int warps[3] = {4, 8, 16};
+  const uint32_t shares[4] = {1, 4, 16, 32}, lines[5] = {2048, 4096, 8192, 16384, 32768};
+  int n = 0;
+  for (int w = 0; w < 3; ++w) {
+    BatchPlan seen[20];
+    int m = 0;
+    for (uint32_t share : shares)
+      for (uint32_t line : lines) {
+        const BatchPlan p = batch_plan(B, sms, (uint32_t)ctas_per_sm[w], warps[w], share * (uint32_t)warps[w], line, true);
+        bool dup = false;
+        for (int i = 0; i < m; ++i)
+          dup = dup || (seen[i].grid == p.grid && seen[i].group == p.group && seen[i].long_bytes == p.long_bytes);
+        if (dup) continue;
+        seen[m++] = p;
+        out[n++] = BatchCandidate{warps[w], share * (uint32_t)warps[w], line};
+      }
+  }
+  return n;
 }
 
 }  // namespace gbu

@@ -18,6 +18,12 @@ extern "C" void plan(uint64_t B, uint32_t sms, uint32_t per_sm, int warps, uint3
   const gbu::BatchPlan p = gbu::batch_plan(B, sms, per_sm, warps, claim, long_bytes, chosen != 0);
   out[0] = p.grid; out[1] = p.group; out[2] = p.per_cta; out[3] = p.long_bytes;
 }
+extern "C" int candidates(uint64_t B, uint32_t sms, int p4, int p8, int p16, uint32_t *out) {
+  gbu::BatchCandidate c[gbu::BATCH_CANDIDATES];
+  const int per_sm[3] = {p4, p8, p16}, n = gbu::batch_candidates(B, sms, per_sm, c);
+  for (int i = 0; i < n; ++i) { out[3 * i] = c[i].warps; out[3 * i + 1] = c[i].claim; out[3 * i + 2] = c[i].long_bytes; }
+  return n;
+}
 """
 SMS = 152
 PER_SM = {4: 8, 8: 4, 16: 2}
@@ -41,6 +47,7 @@ def plan():
         out = (ctypes.c_uint32 * 4)()
         lib.plan(B, SMS, PER_SM[warps], warps, claim, long_bytes, int(chosen), out)
         return dict(zip(("grid", "group", "per_cta", "long_bytes"), out))
+    call.lib = lib
     return call
 
 
@@ -66,3 +73,30 @@ def test_few_strings_get_a_cta_each(plan, warps):
         assert plan(B, warps, long_bytes=4096, chosen=True)["long_bytes"] == 4096
     p = plan(resident + 1, warps)
     assert not p["per_cta"] and p["long_bytes"] == 16384
+
+
+@pytest.mark.parametrize("warps", [4, 8, 16])
+@pytest.mark.parametrize("chosen", [False, True])
+def test_a_warps_share(plan, warps, chosen):
+    """The claim's share where no SM idles, less where one would, the largest in a large batch."""
+    full = 16 if warps == 16 else 32
+    for claim in (1, warps, 4 * warps, 10 * warps, 1024):
+        assert plan(300_000, warps, claim, chosen=chosen)["group"] == max(1, min(full, claim // warps))
+        assert plan(2000, warps, claim, chosen=chosen)["group"] <= max(1, 2000 // SMS // warps)
+        assert plan(10 ** 6, warps, claim, chosen=chosen)["group"] == full
+
+
+@pytest.mark.parametrize("B", [1, 300, 609, 5000, 20000, 10 ** 6])
+def test_the_tuners_candidates_are_distinct_launches(plan, B):
+    out = (ctypes.c_uint32 * 180)()
+    n = plan.lib.candidates(ctypes.c_uint64(B), SMS, PER_SM[4], PER_SM[8], PER_SM[16], out)
+    seen = set()
+    for i in range(n):
+        warps, claim, line = out[3 * i:3 * i + 3]
+        p = plan(B, warps, claim, line, chosen=True)
+        seen.add((warps, p["grid"], p["group"], p["long_bytes"]))
+        assert 1 <= claim <= 1024 and line >= 512
+    assert len(seen) == n
+    if B == 10 ** 6:  # every claim comes to the same launch
+        assert n == 15
+    assert {w for w, *_ in seen} == {4, 8, 16} and {s[3] for s in seen} == {2048, 4096, 8192, 16384, 32768}
