@@ -214,13 +214,6 @@ __device__ __forceinline__ uint4 ldg_stream(const uint8_t *p) {
   return v;
 }
 
-// The same for 32 bytes (p 32-byte aligned)
-__device__ __forceinline__ void ldg32_stream(const uint8_t *p, uint32_t (&w)[8]) {
-  asm volatile("ld.global.nc.L1::no_allocate.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
-               : "l"(p));
-}
-
 __device__ __forceinline__ uint32_t ldg_word(const uint8_t *p) {
   return __ldg(reinterpret_cast<const unsigned int *>(p));
 }

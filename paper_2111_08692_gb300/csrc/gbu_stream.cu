@@ -242,26 +242,29 @@ __global__ void __launch_bounds__(STREAM_THREADS, stream_min_blocks<KMODE>()) st
 }
 
 // UTF-8 validation: a warp streams 4 KiB warp tiles, four regions of 1 KiB, a lane 32 consecutive
-// bytes of each (one 256-bit load; the source base is rounded to 32 bytes), judged on bit planes
-// (gbu_planes.cuh).  A region without a byte >= 80 takes one vote; one without a byte >= E0 is judged
-// four bytes at a time (1 GiB of Latin or Cyrillic: 267 us on the planes, 252 by the byte-wise
-// kernel before them, 221 so), tried only while the warp's last region was such a one (the route
-// costs CJK and emoji 4% even so: 272 to 284 and 290 to 302).  Bound by HBM for ASCII, by the integer
-// pipe else (the planes on CJK: 76% busy, 180 warp instructions per KiB; the byte-wise route before
-// took 280).  Each region's registers are loaded with the warp's next tile as soon as the region is
-// judged, so that three regions' judgement covers the load.  1 GiB of CJK: 440 us by the byte-wise
-// kernel (2.4 TB/s); on the planes alone 266 with all loads of a tile issued together, 261 so.
+// bytes of each (the source base is rounded to 32 bytes), judged on bit planes (gbu_planes.cuh).  A
+// region without a byte >= 80 takes one vote; one without a byte >= E0 is judged four bytes at a
+// time, tried only while the warp's last region was such a one.  Bound by HBM for ASCII, by the
+// integer pipe else.  1 GiB, us (GB300, one sitting): ASCII / Latin / CJK / emoji 150 / 254 / 441 /
+// 531 by the byte-wise kernel before the planes, 150 / 271 / 271 / 289 on the planes alone,
+// 148 / 216 / 278 / 296 with the two-byte route.  The warp's next tile is loaded when all four regions
+// are judged, two 16-byte loads for a lane's 32 bytes: with one 256-bit load as soon as each region
+// was judged, 152 / 218 / 281 / 300, and ASCII right after a kernel that left L2 full of its output
+// 183 instead of 171.
 constexpr int V8_REGIONS = (int)(WT_BYTES / 1024u);
 
 // The lane's 32 bytes at virtual position c (bytes outside the input read as zero).
 __device__ __forceinline__ void load_lane32(const Params &p, long long c, bool inside, uint32_t (&w)[8]) {
+  uint4 a, b;
   if (inside) {
-    ldg32_stream(p.base + c, w);
+    a = ldg_stream(p.base + c);
+    b = ldg_stream(p.base + c + 16);
   } else {
-    const uint4 a = load_chunk(p, c, false), b = load_chunk(p, c + 16, false);
-    w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
-    w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
+    a = load_chunk(p, c, false);
+    b = load_chunk(p, c + 16, false);
   }
+  w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
+  w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
 }
 
 __global__ void __launch_bounds__(STREAM_THREADS, 3) validate8_kernel(const Params p) {
@@ -321,9 +324,10 @@ __global__ void __launch_bounds__(STREAM_THREADS, 3) validate8_kernel(const Para
       } else {
         pending = 0;
       }
-      if (more) load_lane32(p, t1 + 1024 * r + 32 * lane, in, W[r]);
     }
     if (more) {
+#pragma unroll
+      for (int r = 0; r < V8_REGIONS; ++r) load_lane32(p, t1 + 1024 * r + 32 * lane, in, W[r]);
       pre = edge_word(t1 - 4, in);
       post = edge_word(t1 + WT_BYTES, in);
     }
