@@ -52,14 +52,14 @@ def sources_hash() -> str:
 
 
 # The sources each single-buffer kernel is compiled from (its device code), by operation.
-_STREAM = ["gbu_stream.cu", "gbu_planes.cuh", "gbu_chunk.cuh", "gbu_device.cuh"]
+_STREAM = ["gbu_stream.cu", "gbu_planes.cuh", "gbu_chunk.cuh", "gbu_device.cuh", "gbu_grid.h"]
 KERNEL_SOURCES = {
     "validate_utf8": _STREAM, "utf16_length_from_utf8": _STREAM,
     "validate_utf16le": _STREAM, "utf8_length_from_utf16le": _STREAM,
     "convert_utf8_to_utf16le": ["gbu_utf8.cu", "gbu_wide_utf8.cuh", "gbu_wide.cuh", "gbu_codec_utf8.cuh",
-                                "gbu_xcode.cuh", "gbu_chunk.cuh", "gbu_device.cuh"],
+                                "gbu_xcode.cuh", "gbu_chunk.cuh", "gbu_device.cuh", "gbu_grid.h"],
     "convert_utf16le_to_utf8": ["gbu_utf16.cu", "gbu_wide_utf16.cuh", "gbu_wide.cuh", "gbu_codec_utf16.cuh",
-                                "gbu_xcode.cuh", "gbu_chunk.cuh", "gbu_device.cuh"],
+                                "gbu_xcode.cuh", "gbu_chunk.cuh", "gbu_device.cuh", "gbu_grid.h"],
 }
 
 

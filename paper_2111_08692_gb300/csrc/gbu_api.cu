@@ -329,13 +329,11 @@ static int make_params(gbu_ctx *c, int &k, const void *src, uint64_t n, uint32_t
 // what fits on the device at once.
 static int launch(gbu_ctx *c, int k, const gbu::Params &p, gbu_stream stream) {
   DeviceGuard g(c->device);
-  uint64_t grid = (uint64_t)c->num_sms * (uint64_t)c->blocks_per_sm[k];
   const uint64_t useful = is_transcoder(k) ? p.ntiles
                                            : (p.ntiles + gbu::STREAM_THREADS / 32 - 1) / (gbu::STREAM_THREADS / 32);
-  if (useful < grid) grid = useful;
-  if (grid < 1) grid = 1;
+  const uint32_t grid = gbu::launch_grid((uint64_t)c->num_sms * (uint64_t)c->blocks_per_sm[k], useful);
   void *args[] = {(void *)&p};
-  cudaError_t e = cudaLaunchKernel(kernel_ptr(k), dim3((unsigned)grid), dim3(kernel_threads(k)), args,
+  cudaError_t e = cudaLaunchKernel(kernel_ptr(k), dim3(grid), dim3(kernel_threads(k)), args,
                                    kernel_smem(k), (cudaStream_t)stream);
   if (e != cudaSuccess) {
     cudaGetLastError();

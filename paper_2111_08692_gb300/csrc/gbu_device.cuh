@@ -21,6 +21,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "gbu_grid.h"
 #include "gbutf.h"
 
 namespace gbu {
@@ -491,9 +492,9 @@ __device__ __forceinline__ bool fold_and_finish(const Params &p, unsigned long l
 // takes, besides the CTA's units, a count of CTAs and of CTAs with an error, so that its old value
 // tells the last CTA everything (the launch's units in `units`, whether the error key is set in
 // `errors`) without another round trip to L2.  add: the CTA's units (thread 0).  Fields: CTAs from
-// bit 52, CTAs with an error from bit 40 (a grid has fewer than 4096 CTAs), units below (no buffer
-// of the device's memory gives 2^40).
-constexpr int FIN_CTAS = 52, FIN_ERRORS = 40;
+// bit 52, CTAs with an error from bit 40 (launch_grid keeps a grid within both), units below (no
+// buffer that the device can address gives 2^40).
+constexpr int FIN_CTAS = 64 - FIN_CTA_BITS, FIN_ERRORS = FIN_CTAS - FIN_CTA_BITS;
 
 template <int NTH>
 __device__ __forceinline__ bool finish_packed(const Params &p, unsigned long long err_pos, unsigned long long add,

@@ -142,9 +142,7 @@ extern "C" int gbu_convert_utf8_to_utf16le_noalloc(const uint8_t *src, uint64_t 
   p.dshift = (uint32_t)((d & 15) / 2);
   p.cap = cap;
 
-  uint32_t grid = (uint32_t)s.grid;
-  if (p.ntiles < grid) grid = p.ntiles;
-  if (grid < 1) grid = 1;
+  const uint32_t grid = gbu::launch_grid((uint64_t)s.grid, p.ntiles);
   void *args[] = {(void *)&p};
   if (cudaLaunchKernel(gbu::utf8_to_utf16_kernel_ptr(false), dim3(grid), dim3(gbu::XT), args,
                        gbu::utf8_to_utf16_smem_bytes(false), (cudaStream_t)stream) != cudaSuccess) {
