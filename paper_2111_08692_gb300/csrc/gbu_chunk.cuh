@@ -296,9 +296,10 @@ static __device__ __noinline__ void resolve_utf8_error(const uint8_t *s, uint64_
   *off = chunk < 0 ? 0 : (uint64_t)chunk;
 }
 
-// UTF-16: a word is flagged exactly when it is the first word of an ill-formed sequence, so
-// the first error lies in the flagged chunk [chunk, chunk + 8).  BE: the words lie in memory
-// with their bytes in big-endian order.
+// UTF-16: a chunk (8 words, or 16 of a wide lane) is flagged when it holds an ill-formed sequence's
+// first word, and by some routes also when the word right after it is an unpaired second surrogate,
+// so the first error lies in the smallest flagged chunk or is the word after it.  BE: the words lie
+// in memory with their bytes in big-endian order.
 template <bool BE = false>
 static __device__ __noinline__ void resolve_utf16_error(const uint16_t *s, uint64_t n, long long chunk,
                                                         uint64_t *off) {

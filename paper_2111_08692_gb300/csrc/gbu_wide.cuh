@@ -339,8 +339,10 @@ __device__ __forceinline__ void wtranscode(const Params &p, WSmem<Codec, R> &sm,
   // Early exit: output past the first error is unspecified, so a CTA stops at a partition that
   // starts past a chunk some thread already flagged (the error key, published at once): later
   // partitions, if anyone still works on them, need no more than the aggregates it has published
-  // for that partition and the next.  The first error lies at most 31 bytes past the smallest
-  // flagged chunk, so it is always converted up to its start.
+  // for that partition and the next.  The smallest flagged chunk is the lane's that holds the first
+  // error, or the one right after it (a cut UTF-8 sequence) or before it (a second surrogate without
+  // a first one, which may then start the next partition).  So whatever the valid prefix holds lies
+  // in partitions that do not start past that chunk, and those are all converted.
   unsigned long long published = NO_ERROR;
   while (cur < p.ntiles) {
     // claim and count the next partition, so that its aggregate is out a partition early

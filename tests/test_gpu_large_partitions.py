@@ -201,3 +201,29 @@ def test_a_wait_that_runs_out(large):
         large.codec.set_wait_limit(1 << 22)
     assert r[0] == "TIMEOUT"
     large.check()
+
+
+@pytest.mark.parametrize("size", [3 * PART, None], ids=["4KiB", "16KiB"])
+@pytest.mark.parametrize("be", [False, True])
+def test_second_surrogate_first_in_a_partition(codec, size, be):
+    """An unpaired second surrogate that is the first word of a partition, after a region with pairs: the
+    last lane of that region flags it, in the partition before the one it lies in, so that with early exit
+    the latter may be left out; the result is the same."""
+    import torch
+    from paper_2111_08692_gb300 import result_tuple
+    large = Large(torch, codec, True, be)
+    part = 4096 if size else PART
+    for at in (part // 2, part, 4 * part // 2):
+        pairs = np.tile(np.array([0xD83D, 0xDE00], np.uint16), at // 2)
+        head = np.concatenate([pairs, np.array([0xDC00, 0x41], np.uint16), pairs[:600]])
+        for early in (True, False):
+            if size is None:
+                large.check(head, early=early)
+                continue
+            codec.set_early_exit(early)
+            src = large._dev(head)
+            dst = torch.zeros(3 * head.size, dtype=torch.uint8, device="cuda")
+            assert result_tuple(large.call(src, dst)) == ("SURROGATE", at)
+            out = torch.from_numpy(oracle.convert_utf16le_to_utf8(pairs)[1].copy()).cuda()
+            assert torch.equal(dst[:out.numel()], out)
+            codec.set_early_exit(True)
