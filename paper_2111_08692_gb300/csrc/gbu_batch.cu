@@ -5,17 +5,17 @@
 // code units) or as an array of descriptors (pointer and length of each input and output).
 // In a persistent grid of CTAs (NWARPS warps each)
 //   * every warp claims groups of up to 32 consecutive strings (a counter in the workspace) and
-//     packs them: the strings' 16-byte chunks are numbered back to back, a lane takes one chunk, and a warp step
-//     handles 32 of them, whatever strings they belong to.  Segmented scans give each string its
+//     packs them: the strings' 16-byte chunks are numbered back to back, a lane takes one chunk,
+//     and a warp step handles 32 of them, whatever strings they belong to.  Segmented scans give each string its
 //     length, its first error and its place in the output.  A warp step on one string at a time
 //     left most lanes idle (half of a log-normal column's strings have under 64 bytes, four
 //     lanes' worth): 522 to 1427 warp instructions per string of 197 bytes on average, now 109
 //     to 393.  A million such strings, lengths, scan and conversion in both directions: 4,421 us
-//     before, 1,113 us now (GB300);
+//     before, 1,088 us now (GB300);
 //   * a string of at least long_bytes input bytes is set aside and handled by the whole CTA once
-//     its warps find no more groups (or its list of them fills up): NWARPS 512-byte regions per step (one 16-byte chunk per lane): for a transcoding
-//     each warp counts its region first and the CTA scans the counts, so every region knows where
-//     its output starts.
+//     its warps find no more groups (or its list of them fills up): NWARPS 512-byte regions per
+//     step (one 16-byte chunk per lane); for a transcoding each warp counts its region first and the
+//     CTA scans the counts, so every region knows where its output starts.
 // The chunks' analysis is that of the single-buffer kernels, so each string's result is the one a
 // single-buffer call on it gives.
 // A batch of no more strings than resident CTAs gives each a CTA of its own (gbu_batch_plan.h).
@@ -23,8 +23,8 @@
 // from the caller's dst_off (for example the exclusive scan of the batched lengths).
 // What bounds it: instruction issue on the integer pipe (63-65% busy in the conversions), then the
 // latency of a step's loads, which are issued a step ahead.
-// The launch geometry (warps per CTA, strings per claim, long-string threshold) is chosen by
-// the library's autotuner from timed candidates.
+// The launch geometry (warps per CTA, strings per claim, long-string threshold) is the library's, the
+// caller's or the autotuner's, which times candidates.
 #include <stdint.h>
 
 #include "gbu_batch_plan.h"
@@ -655,7 +655,8 @@ __device__ __forceinline__ void cta_string(const BatchParams &bp, uint64_t i, Ba
 }
 
 // Resident warps per SM the register budget is held to: 32 (64 registers a thread), 24 for the
-// UTF-8 -> UTF-16 transcoder (80).  FEW: CTA i handles string i and nothing else, together or with its
+// UTF-8 -> UTF-16 transcoder (80); its CTAs of 16 warps do not share an SM then, so they get up to 128
+// registers for 16 resident warps (a million strings: 395 us, with 8 warps 377).  FEW: CTA i handles string i and nothing else, together or with its
 // first warp (an instance of its own: the same test inside the claim loop spilled more registers there,
 // and a million strings took 1,090 us instead of 1,084).
 template <int MODE, int NWARPS, bool FEW>

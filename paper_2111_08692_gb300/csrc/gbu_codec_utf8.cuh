@@ -267,14 +267,6 @@ struct Utf8ToUtf16 {
                                                           long long c, bool edge, uint16_t *st, uint32_t base,
                                                           uint32_t x0, uint32_t rtot, unsigned long long err_pos,
                                                           uint32_t stage) {
-    return convert_general_body(lo, hi, v, prev, next, c, edge, st, base, x0, rtot, err_pos, stage);
-  }
-
-  // The body of convert_general, for callers that inline it.
-  __device__ __forceinline__ static General convert_general_body(long long lo, long long hi, uint4 v, uint32_t prev,
-                                                                 uint32_t next, long long c, bool edge, uint16_t *st,
-                                                                 uint32_t base, uint32_t x0, uint32_t rtot,
-                                                                 unsigned long long err_pos, uint32_t stage) {
     uint32_t W[6];
     W[0] = prev;
     W[1] = v.x; W[2] = v.y; W[3] = v.z; W[4] = v.w;

@@ -3,8 +3,8 @@
 // Two kernel shapes:
 //   * read-only kernels (validation, lengths; gbu_stream.cu) stream 4 KB warp tiles with
 //     16-byte loads, never waiting on another CTA;
-//   * transcoders (gbu_utf8.cu, gbu_utf16.cu) walk 16 KB partitions claimed from a ticket
-//     counter.  A CTA counts the output units of partition k+1 (a read from HBM) and
+//   * transcoders (gbu_utf8.cu, gbu_utf16.cu and their kin) walk 16 KiB partitions, or 4 KiB ones
+//     of a small input (gbu_wide.cuh), claimed from a ticket counter.  A CTA counts the output units of partition k+1 (a read from HBM) and
 //     publishes that aggregate before it transcodes partition k (a re-read, normally from
 //     L2).  Partition k's output offset comes from the single-pass decoupled look-back of
 //     Merrill & Garland ("Single-pass Parallel Prefix Scan with Decoupled Look-back", 2016):
@@ -52,17 +52,19 @@ constexpr unsigned long long NO_ERROR = ~0ull;
 struct WsHeader {
   uint32_t epoch;                 // tags scan states of the current launch (1 .. 2^18-1)
   uint32_t ticket;                // next partition to claim (transcoders)
-  uint32_t done;                  // CTAs that have finished
+  uint32_t done;                  // CTAs that have finished (kernels without the packed completion)
   uint32_t status;                // sticky: 1 = a wait gave up (GBU_TIMEOUT)
   unsigned long long errkey;      // smallest input position of a thread chunk with an error
-  unsigned long long total;       // sum of partition aggregates (output length)
+  unsigned long long total;       // sum of partition aggregates (output length); with the packed
+                                  // completion also the counts of CTAs (finish_packed)
   uint32_t stop_tile;             // validation early exit: smallest warp tile with a flagged chunk
   uint32_t pad[23];
 };
 static_assert(sizeof(WsHeader) == 128, "header is one 128-byte line");
 
 struct Params {
-  const uint8_t *base;     // source rounded down to 16 bytes
+  const uint8_t *base;     // source rounded down to 16 bytes; to 32 for the wide transcoders, whose
+                           // 256-bit loads need it, and UTF-8 validation (32 bytes per lane)
   uint64_t vbytes;         // off0 + source bytes: virtual positions [off0, vbytes) are data
   uint32_t off0;           // source address - base (bytes)
   uint32_t ntiles;         // warp tiles (read-only kernels) or partitions (transcoders)

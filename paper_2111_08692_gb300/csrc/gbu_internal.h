@@ -14,7 +14,7 @@ int gbu_internal_batch_desc(gbu_ctx *ctx, int op, const gbu::StringDesc *desc, u
                             gbu_stream stream);
 
 // Launch partitions of a string of n code units at src for transcoding op
-// (GBU_OP_CONVERT_*): its 64 KiB partitions, counting the three positions past the end that
+// (GBU_OP_CONVERT_*): its 16 KiB partitions, counting the three positions past the end that
 // UTF-8 validation judges.
 int gbu_internal_partitions(int op, const void *src, uint64_t n);
 

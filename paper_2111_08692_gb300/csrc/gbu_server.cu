@@ -11,8 +11,8 @@
 //      server's device arena (worst-case size: n words for UTF-8 -> UTF-16LE, 3n bytes for
 //      UTF-16LE -> UTF-8);
 //   3. dispatches admitted requests into free launch-group slots: small requests of one
-//      operation go together into ONE batched launch over device descriptors (warp per
-//      string, CTA per longer string); requests of at least large_bytes each get a
+//      operation go together into ONE batched launch over device descriptors (few strings: a
+//      CTA each); requests of at least large_bytes each get a
 //      single-buffer launch (all SMs on one string), several per group.  A group is: the
 //      launches and an event.  Its descriptors and results either stay in mapped pinned host
 //      memory, which the kernels read and write directly over the host link, or (device_rings)

@@ -7,9 +7,9 @@
 //     a UTF-32 input, the UTF-32 length of a UTF-8 or UTF-16LE input), streaming 4 KB warp tiles
 //     like the UTF-8 and UTF-16 read-only kernels; a unit needs no neighbour.
 //   * utf32_to_utf8_kernel / utf8_to_utf32_kernel: the partition loop of gbu_xcode.cuh with the
-//     two codecs below.  UTF-32 -> UTF-8 encodes each unit in 1-4 bytes; UTF-8 -> UTF-32 checks
-//     rules 1-6 with the word-level tests of gbu_chunk.cuh and stores one unit per leading byte,
-//     decoded from the four bytes that start there.
+//     two codecs below.  UTF-32 -> UTF-8 encodes each unit in 1-4 bytes, without a branch per unit;
+//     UTF-8 -> UTF-32 runs the byte-plane body of the UTF-8 -> UTF-16 transcoder
+//     (gbu_wide_utf8.cuh), which checks rules 1-6, and stores one unit per leading byte.
 //   * utf32_to_utf16_kernel / utf16_to_utf32_kernel: the same loop between UTF-16LE and UTF-32:
 //     a unit becomes one word (below 0x10000) or a surrogate pair; a UTF-16 word that is not a
 //     second surrogate becomes one unit (a first surrogate with its partner, which may be the

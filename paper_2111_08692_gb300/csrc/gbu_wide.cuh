@@ -2,8 +2,7 @@
 // 32 input bytes per lane and 1 KiB warp regions.
 //
 // The loop has the shape of gbu_xcode.cuh's: a CTA of XT threads claims partitions of R x 4 KiB
-// (16 KiB, or 4 KiB for small inputs: see WIDE_SMALL_BYTES) from
-// a ticket counter, counts the output of the NEXT partition (a read from HBM) and publishes
+// (16 KiB, or 4 KiB for small inputs: see wide_small_bytes) from a ticket counter, counts the output of the NEXT partition (a read from HBM) and publishes
 // that aggregate before it takes the CURRENT partition's output offset from the CTA-wide
 // decoupled look-back, then converts the current partition (a re-read, normally from L2)
 // through per-warp staging buffers and bulk stores.  What differs is the grain, chosen so that
@@ -55,8 +54,8 @@ static_assert(SLICE_BYTES == WREGION * WROUNDS, "a slice is whole regions");
 __host__ __device__ constexpr uint32_t wide_part_bytes(int R) { return (uint32_t)(R * XWARPS) * WREGION; }
 // Small inputs run on partitions of one region per warp (4 KiB): four times as many CTAs share the
 // work, and a warp converts one region instead of four in a row.  The line lies at one and a half
-// such partitions per resident CTA (7.5 MB on 152 SMs); past it the fixed work per partition
-// counts.  Mixed text, 4 KiB / 16 KiB partitions, us per launch (GB300), 8 -> 16: 4 KB 7.7 / 19.5,
+// such partitions per resident CTA (7.5 MB on 152 SMs), where 16 -> 8 crosses over: past it the fixed
+// work per partition counts.  8 -> 16 crosses over later, past 16 MiB; one line serves both.  Mixed text, 4 KiB / 16 KiB partitions, us per launch (GB300), 8 -> 16: 4 KB 7.7 / 19.5,
 // 1 MiB 10.1 / 23.7, 4 MiB 15.6 / 24.0, 6 MiB 21.3 / 25.6, 16 MiB 36.0 / 39.2; 16 -> 8: 4 KB 10.5 /
 // 17.9, 1 MiB 12.7 / 21.2, 4 MiB 18.9 / 22.5, 8 MiB 28.2 / 28.5, 16 MiB 44.7 / 42.3.
 __host__ __device__ constexpr uint64_t wide_small_bytes(uint64_t ctas) { return ctas * wide_part_bytes(1) * 3 / 2; }

@@ -4,12 +4,12 @@
 // Paper Section 3: words 0000-D7FF and E000-FFFF are characters by themselves; a word in
 // D800-DBFF must be followed by one in DC00-DFFF and the pair encodes
 // ((first & 0x3FF) << 10 | (second & 0x3FF)) + 0x10000.  The UTF-8 sizes are 1 byte below
-// 0x80, 2 below 0x800, 3 otherwise, and 2 per surrogate word (a pair's first word writes all 4
-// bytes, over its own 2 slots and its partner's).  Section 4 routes whole registers by range;
+// 0x80, 2 below 0x800, 3 otherwise, and 2 per surrogate word, which writes its own two of its pair's
+// four.  Section 4 routes whole registers by range;
 // here the routes are taken per warp region from the count pass's flags: all ASCII (words
 // narrowed to bytes), one and two bytes, no surrogates, ASCII and pairs only (emoji-heavy
-// text), and the general pair route.  Words are encoded one at a time into the warp's staging
-// buffer through 32-bit shared-memory addresses.
+// text), and the general pair route.  All but the first encode two words per 32-bit register and
+// store the bytes into the warp's staging buffer through 32-bit shared-memory addresses.
 #pragma once
 
 #include <stdint.h>
