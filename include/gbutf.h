@@ -250,8 +250,8 @@ int gbu_per_string_loop(gbu_ctx *ctx, int op, const void *src, const uint64_t *o
  * x 512 bytes per step).  strings_per_claim is a wish: in a batch that would leave SMs idle the share
  * is smaller, and in one that gives every resident warp four times the largest share (about 600,000
  * strings) it is the largest.  A batch of no more strings than the device runs CTAs at
- * once has a CTA for each string, and then, unless the geometry was set or tuned, strings of 1536
- * bytes on are handled by their whole CTA. */
+ * once has a CTA for each string, and then, unless the geometry was set or was tuned on such a
+ * batch, strings of 1536 bytes on are handled by their whole CTA. */
 typedef struct {
   int32_t warps_per_cta;      /* 4, 8 or 16 (default 8) */
   uint32_t strings_per_claim; /* 1 .. 1024 (default 64) */
@@ -263,7 +263,7 @@ int gbu_get_batch_config(const gbu_ctx *ctx, int op, gbu_batch_config *cfg);
 int gbu_set_batch_config(gbu_ctx *ctx, int op, const gbu_batch_config *cfg); /* checks ranges */
 /* Autotuner: runs operation `op` on the given batch (arguments as for the batched call of
  * that operation; `out` is results or lens) for each candidate geometry (warps 4/8/16 x
- * claims of 1/4/16/32 strings per warp x long-string thresholds of 2/4/8/16/32 KiB, without those
+ * claims of 32/16/4/1 strings per warp x long-string thresholds of 2/4/8/16/32 KiB, without those
  * that come to the same launch on this batch), one untimed and
  * `reps` timed launches each (CUDA events on `stream`), keeps the fastest in the context and
  * writes it to *chosen (may be NULL).  The last launch uses the chosen geometry, so the

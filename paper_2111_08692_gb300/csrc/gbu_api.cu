@@ -115,7 +115,7 @@ struct gbu_ctx {
   int scan_blocks_per_sm;
   int seg_blocks_per_sm[2];             // several-string transcoders: 8 -> 16, 16 -> 8
   gbu_batch_config batch_cfg[K_COUNT];  // launch geometry of the batched kernels
-  bool batch_chosen[K_COUNT];           // set by the caller or the tuner
+  bool batch_chosen[K_COUNT];           // set by the caller, or by the tuner on few strings
   std::atomic<uint64_t> launches;
   uint64_t capture_start;               // launches when the current graph capture began
 };
@@ -684,7 +684,7 @@ static int batch_check_config(const gbu_batch_config &b) {
   return GBU_OK;
 }
 
-// Launches batched mode m over B strings with geometry cfg (chosen: not the library's defaults).
+// Launches batched mode m over B strings with geometry cfg (chosen: as batch_plan takes it).
 static int batch_launch(gbu_ctx *c, int m, const gbu_batch_config &cfg, bool chosen, const void *src,
                         const uint64_t *off, uint64_t B, void *dst, const uint64_t *dst_off, gbu_result *results,
                         uint64_t *lens, gbu_stream stream, const gbu::StringDesc *desc = nullptr) {
@@ -867,7 +867,11 @@ extern "C" int gbu_tune_batched(gbu_ctx *c, int op, const void *src, const uint6
   if (rc == GBU_OK) {
     best.tuned_ms = best_ms;
     c->batch_cfg[op] = best;
-    c->batch_chosen[op] = true;
+    // a threshold found on a large batch says nothing about few strings (and the other way round it is
+    // the caller's wish)
+    c->batch_chosen[op] =
+        gbu::batch_plan(B, (uint32_t)c->num_sms, (uint32_t)c->batch_blocks_per_sm[op][warps_index(best.warps_per_cta)],
+                        best.warps_per_cta, best.strings_per_claim, best.long_bytes, true).per_cta;
     rc = batch_launch(c, op, best, true, src, off, B, dst, dst_off, results, lens, stream);
     if (rc == GBU_OK && cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) rc = GBU_CUDA_ERROR;
   }

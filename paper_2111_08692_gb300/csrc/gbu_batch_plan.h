@@ -22,8 +22,8 @@ struct BatchPlan {
 };
 
 // B strings (B >= 1) on a device with `sms` SMs and `ctas_per_sm` resident CTAs of `warps` warps each.
-// claim, long_bytes: the context's geometry; chosen: set by the caller or the tuner (else the
-// library's defaults).
+// claim, long_bytes: the context's geometry; chosen: long_bytes was set by the caller, or by the tuner
+// on few strings, and holds for few strings too.
 inline BatchPlan batch_plan(uint64_t B, uint32_t sms, uint32_t ctas_per_sm, int warps, uint32_t claim,
                             uint32_t long_bytes, bool chosen) {
   const uint32_t full = batch_group_max(warps);
@@ -65,11 +65,12 @@ struct BatchCandidate {
 constexpr int BATCH_CANDIDATES = 60;
 
 // The geometries that the tuner times on a batch of B strings, without those that come to the launch of
-// an earlier one: warps 4, 8 and 16, a warp's share of a claim 1, 4, 16 and 32 strings, and long strings
-// from 2 to 32 KiB.  ctas_per_sm: resident CTAs per SM for 4, 8 and 16 warps.  Returns their number.
+// an earlier one: warps 4, 8 and 16, a warp's share of a claim 32, 16, 4 and 1 strings (the largest
+// first: of claims that are one launch here, the largest is the one to keep for other batches), and long
+// strings from 2 to 32 KiB.  ctas_per_sm: resident CTAs per SM for 4, 8 and 16 warps.  Returns their number.
 inline int batch_candidates(uint64_t B, uint32_t sms, const int (&ctas_per_sm)[3], BatchCandidate (&out)[BATCH_CANDIDATES]) {
   const int warps[3] = {4, 8, 16};
-  const uint32_t shares[4] = {1, 4, 16, 32}, lines[5] = {2048, 4096, 8192, 16384, 32768};
+  const uint32_t shares[4] = {32, 16, 4, 1}, lines[5] = {2048, 4096, 8192, 16384, 32768};
   int n = 0;
   for (int w = 0; w < 3; ++w) {
     BatchPlan seen[20];
