@@ -208,9 +208,12 @@ extern "C" gbu_ctx *gbu_create(int device, uint64_t max_units) {
   bool occ_ok = true;
   for (int m = 0; m < K_COUNT && occ_ok; ++m)
     for (int w = 0; w < 3 && occ_ok; ++w) {
-      int bps = 0;
+      int bps = 0, few = 0;
+      // (the instance for few strings is asked too, so that its first launch loads nothing)
       occ_ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, gbu::batch_kernel_ptr(m, kWarps[w], false),
-                                                             kWarps[w] * 32, 0) == cudaSuccess && bps >= 1;
+                                                             kWarps[w] * 32, 0) == cudaSuccess && bps >= 1 &&
+               cudaOccupancyMaxActiveBlocksPerMultiprocessor(&few, gbu::batch_kernel_ptr(m, kWarps[w], true),
+                                                             kWarps[w] * 32, 0) == cudaSuccess && few >= 1;
       c->batch_blocks_per_sm[m][w] = bps;
     }
   occ_ok = occ_ok && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c->scan_blocks_per_sm, gbu::scan_kernel_ptr(),
